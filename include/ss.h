@@ -271,7 +271,9 @@ ss_status ss_batch_create(ss_ctx* const* ctxs, int32_t nctx, const ss_batch_item
  * launches, or 0: merged lanes (each chunk a host thread with its own stream;
  * the transforms of all lanes, of rings N >= 8192, run together as one
  * persistent launch per phase over all their tiles); ntt_tile_log: 11 or 12
- * (words per transform tile). Kernel timing does not cover merged lanes. */
+ * (words per transform tile, for rings N >= 8192 on primes of more than 55
+ * bits; other transforms have one tile size). Kernel timing does not cover
+ * merged lanes. */
 ss_status ss_batch_config(ss_batch* b, int32_t chunk, int32_t nstreams, int32_t ntt_tile_log);
 ss_status ss_batch_get_config(const ss_batch* b, int32_t* chunk, int32_t* nstreams, int32_t* ntt_tile_log,
                               int32_t* groups, int32_t* skipped);

@@ -122,7 +122,6 @@ struct LaneMerger : NttMerger, KsMerger {
   cudaStream_t mst = nullptr;
   cudaEvent_t done = nullptr;
   std::vector<cudaEvent_t> lane_ev;
-  int tile_log = SS_NTT_TILE_LOG;
   bool failed = false;
   std::string error;
 
@@ -138,8 +137,8 @@ struct LaneMerger : NttMerger, KsMerger {
         if (q.ks) ks.push_back(q.k);
         else (q.fwd ? fw : iv).push_back(q.r);
       }
-      ntt_multi(fw, true, tile_log, mst);
-      ntt_multi(iv, false, tile_log, mst);
+      ntt_multi(fw, true, mst);
+      ntt_multi(iv, false, mst);
       ks_multi(ks, mst);
       SS_CUDA(cudaEventRecord(done, mst));
       for (auto& q : pending) SS_CUDA(cudaStreamWaitEvent(q.st, done, 0));
@@ -216,7 +215,6 @@ static void run_lanes(ss_batch& b, cudaStream_t st) {
   LaneMerger M;
   M.active = n;
   M.mst = b.streams[n];
-  M.tile_log = b.tile_log;
   M.done = b.events[n + 1];
   for (int k = 0; k < n; ++k) M.lane_ev.push_back(b.events[k]);
   cudaEvent_t fork = b.events[n];

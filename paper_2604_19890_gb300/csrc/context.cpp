@@ -532,6 +532,7 @@ static void upload(void** dst, const void* src, size_t bytes) {
 Context::~Context() {
   cudaFree(d_mod);
   cudaFree(d_tw);
+  cudaFree(d_tp);
   cudaFree(d_ninv);
   cudaFree(d_r64);
   cudaFree(d_split);
@@ -644,22 +645,38 @@ void build_context(Context& C, const ss_params& prm) {
 
   // twiddles: psi^brv(i) and psi^-brv(i) with Shoup companions (m = 2N; m = 3N below)
   {
-    std::vector<u64> tw((size_t)T * 4 * N);
-    std::vector<u64> ninv(4 * T), pinv(2 * T), r64(4 * T, 0);
+    // transforms of N >= 8192 multiply by halves where the primes leave nine spare bits
+    const bool halves = N >= 8192 && prm.bits <= 55;
+    const size_t slots = halves ? ntt_tw_slots(C) : N;  // per prime and direction
+    std::vector<u64> tw((size_t)T * 4 * slots);
+    std::vector<int> slot(halves ? N : 0);
+    for (int k = 1; k < N && halves; ++k) slot[k] = ntt_tw_slot(C, k);
+    std::vector<u32> tp(halves ? (size_t)T * 4 * slots : 0);
+    std::vector<u64> ninv(6 * T, 0), pinv(2 * T), r64(4 * T, 0);
     std::vector<u64> split(C.m_odd == 5 ? (size_t)T * 24 : 0);
     for (int i = 0; i < T; ++i) {
       u64 q = C.primes[i], ps = C.psi[i], pi = nt::inv(ps, q);
       r64[4 * i] = (UINT64_MAX % q + 1) % q;  // 2^64 mod q
-      u64* o = &tw[(size_t)i * 4 * N];
-      auto put = [&](int k, u64 f, u64 bk) {
-        o[2 * k] = f;
-        o[2 * k + 1] = nt::shoup(f, q);
-        o[2 * N + 2 * k] = bk;
-        o[2 * N + 2 * k + 1] = nt::shoup(bk, q);
+      u64* o = &tw[(size_t)i * 4 * slots];
+      auto put = [&](int node, u64 f, u64 bk) {
+        const size_t k = halves && node > 0 ? slot[node] : node;
+        for (int dir = 0; dir < 2; ++dir) {
+          const u64 w = dir ? bk : f;
+          const size_t at = dir * 2 * slots + 2 * k;
+          const u64 s = nt::shoup(w, q);  // floor(w 2^64 / q)
+          o[at] = w;
+          o[at + 1] = s;
+          if (halves) {
+            // s = (s >> 32) 2^32 + low: w_1 = 2^32 w - (s >> 32) q, and floor(w_1 2^32 / q) is s's low word
+            o[at + 1] = (w << 32) - (s >> 32) * q;
+            tp[(size_t)i * 4 * slots + at] = (u32)(s >> 33);
+            tp[(size_t)i * 4 * slots + at + 1] = (u32)s >> 1;
+          }
+        }
       };
       u64 ni = nt::inv((u64)N % q, q);
-      ninv[4 * i] = ni;
-      ninv[4 * i + 1] = nt::shoup(ni, q);
+      ninv[6 * i] = ni;
+      ninv[6 * i + 1] = nt::shoup(ni, q);
       if (C.m_odd == 5) {
         // Phi_m = prod_h (X^(N/4) - x_h), x_h = xi^(e_h), xi = omega^(N/4), e =
         // (1, 3, 7, 9): nodes 1..3 are replaced by the four-way split (table
@@ -691,8 +708,6 @@ void build_context(Context& C, const ss_params& prm) {
           sp[2 * k2] = vals[k2];
           sp[2 * k2 + 1] = nt::shoup(vals[k2], q);
         }
-        ninv[4 * i + 2] = 0;
-        ninv[4 * i + 3] = 0;
       } else if (C.m_odd == 3) {
         // Phi_3N = (X^(N/2) - rho)(X^(N/2) - rho^5), rho = omega^(N/2): node 1
         // is that split (forward twiddle rho; the inverse recovers the high
@@ -706,7 +721,7 @@ void build_context(Context& C, const ss_params& prm) {
         for (u64 e = 1; e < m; ++e) pw[e] = nt::mul(pw[e - 1], ps, q);
         const u64 rho = pw[N / 2];
         const u64 wb = nt::inv((2 * rho + q - 1) % q, q);
-        put(0, 1, nt::mul(wb, ni, q));  // inverse word 0: (2 rho - 1)^-1 N^-1 for the fused last stage
+        put(0, 1, 1);
         put(1, rho, wb);
         for (int k = 2; k < N; ++k) {
           const int l = 31 - __builtin_clz((unsigned)k);
@@ -717,8 +732,10 @@ void build_context(Context& C, const ss_params& prm) {
         }
         // the fused last inverse stage's difference output: 2 (2 rho - 1)^-1 N^-1
         const u64 c1 = nt::mul(2 % q, nt::mul(wb, ni, q), q);
-        ninv[4 * i + 2] = c1;
-        ninv[4 * i + 3] = nt::shoup(c1, q);
+        ninv[6 * i + 2] = c1;
+        ninv[6 * i + 3] = nt::shoup(c1, q);
+        ninv[6 * i + 4] = nt::mul(wb, ni, q);
+        ninv[6 * i + 5] = nt::shoup(ninv[6 * i + 4], q);
       } else {
         std::vector<u64> fw(N), bw(N);
         u64 a = 1, b = 1;
@@ -734,14 +751,15 @@ void build_context(Context& C, const ss_params& prm) {
         r64[4 * i + 3] = nt::mul(r64[4 * i + 2], bw[N / 2], q);
         // N^-1 times the last inverse stage's twiddle psi^-bitrev(1) = psi^(-N/2)
         const u64 wni = nt::mul(ni, bw[N / 2], q);
-        ninv[4 * i + 2] = wni;
-        ninv[4 * i + 3] = nt::shoup(wni, q);
+        ninv[6 * i + 2] = wni;
+        ninv[6 * i + 3] = nt::shoup(wni, q);
       }
       u64 pv = nt::inv((u64)C.p % q, q);
       pinv[2 * i] = pv;
       pinv[2 * i + 1] = nt::shoup(pv, q);
     }
     upload((void**)&C.d_tw, tw.data(), tw.size() * 8);
+    if (halves) upload((void**)&C.d_tp, tp.data(), tp.size() * 4);
     upload((void**)&C.d_ninv, ninv.data(), ninv.size() * 8);
     upload((void**)&C.d_r64, r64.data(), r64.size() * 8);
     if (C.m_odd == 5) upload((void**)&C.d_split, split.data(), split.size() * 8);

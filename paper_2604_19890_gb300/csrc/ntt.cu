@@ -10,16 +10,25 @@
 //
 // A length-N transform is split N = N1 * N2. Its first log2(N1) stages act on
 // the N2 columns (stride N2) independently, the remaining log2(N2) stages on
-// the N1 contiguous chunks of N2 words. Each phase is one kernel: a CTA
-// stages a tile of CPB columns (or chunks) in shared memory (32 KiB), runs
-// its stages there with Harvey lazy butterflies (residues in [0, 4q) forward,
-// [0, 2q) inverse) and writes the tile back. N <= 4096 runs in one phase.
+// the N1 contiguous chunks of N2 words. Each phase is one kernel whose CTAs hold
+// 2048-word tiles in registers and shared memory. N <= 4096 runs in one phase.
+// Three forms, by size and prime width:
+//  * N >= 8192, primes below 2^55: k_ntt16_cols / k_ntt16_rows (products by
+//    halves, below). One GB300, 328 limbs of 2^16 words: 0.565 us a limb forward
+//    and 0.573 inverse, where the Shoup form takes 0.751 and 0.870.
+//  * N >= 8192, wider primes: k_ntt16 (Shoup products: halves need nine spare bits).
+//  * N <= 4096: k_ntt, one phase in shared memory with Harvey's lazy butterflies.
 #include "modarith.cuh"
 #include "ss_internal.h"
 
 namespace ss {
 
 namespace {
+
+__device__ __forceinline__ void cp16(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
 
 constexpr int TILE = 4096;  // words per CTA tile (32 KiB of shared memory)
 
@@ -33,6 +42,19 @@ constexpr int TILE = 4096;  // words per CTA tile (32 KiB of shared memory)
 #ifndef SS_NTT_MINB_I
 #define SS_NTT_MINB_I 3
 #endif
+// resident CTAs of 128 threads per SM that the phases of products by halves are compiled for
+#ifndef SS_COLS_F
+#define SS_COLS_F 7
+#endif
+#ifndef SS_COLS_I
+#define SS_COLS_I 7
+#endif
+#ifndef SS_ROWS_F
+#define SS_ROWS_F 7
+#endif
+#ifndef SS_ROWS_I
+#define SS_ROWS_I 7
+#endif
 #ifndef SS_NTT_MINB_R5
 #define SS_NTT_MINB_R5 3  // m = 5N/2 column phases (the factored split fits the same 80 registers)
 #endif
@@ -43,8 +65,10 @@ struct NttArgs {
   int n_outer, nl, q0, nq, L, N;
   int skip_w, skip_mod, skip_level;
   const Modulus* mods;
-  const u64* tw;     // per prime 4N words: (w, w') pairs forward, then inverse
-  const u64* ninv;   // per prime (N^-1, shoup, N^-1 psi^(-N/2), shoup)
+  const u64* tw;     // per prime 4N words: twiddle word pairs forward, then inverse ((w, w') or (w_0, w_1), TwRow)
+  const u32* tp;     // products by halves: the half-quotients (p_0, p_1) beside A.tw's pairs; else null
+  int tws;           // products by halves: slots per prime and direction, N + N1 (half_tw)
+  const u64* ninv;   // per prime (N^-1, shoup, N^-1 psi^(-N/2), shoup, m = 3N: (2 rho - 1)^-1 N^-1, shoup)
   const u64* split;  // m = 5N/2: per prime 12 (value, shoup) pairs of the four-way split (split4_fwd/inv)
   const u64* src;    // out-of-place first phase: polynomial (o, i) is read at src + o src_os + i N
   long src_os;
@@ -86,6 +110,30 @@ __device__ __forceinline__ int swz16(int lin) {
   return lin ^ ((lin >> 4) & 15);
 }
 
+// Slot of node `widx` of a stage of half-distance 2^logt. In the round of
+// spacing 1 neighbouring threads hold neighbouring groups G of 16 words, and a
+// stage of half-distance below 8 has 2^(3 - logt) twiddles per group: stored
+// group by group, one load of a warp would touch a line per thread (340
+// wavefronts of the L1 path a round and warp, which then bounded the chunk
+// phases at 90 % of its rate). So those stages store, for each block of 2^wb
+// groups, first every group's first twiddle, then every group's second, and so on.
+__host__ __device__ __forceinline__ int tw_slot(int widx, int logt, int wb) {
+  if (logt >= 3) return widx;
+  const int g = widx >> (3 - logt), i = widx & ((1 << (3 - logt)) - 1);
+  return ((g >> wb) << (wb + 3 - logt)) + (i << wb) + (g & ((1 << wb) - 1));
+}
+
+// Tables of products by halves, per prime and direction: slots [0, N1) hold the
+// column phase's nodes, slots N1 + c N2 + l node l of chunk c's own subtree.
+template <bool FWD>
+__device__ __forceinline__ const ulonglong2* half_tw(const NttArgs& A, int pidx) {
+  return reinterpret_cast<const ulonglong2*>(A.tw) + (size_t)(2 * pidx + (FWD ? 0 : 1)) * A.tws;
+}
+template <bool FWD>
+__device__ __forceinline__ const uint2* half_tp(const NttArgs& A, int pidx) {
+  return reinterpret_cast<const uint2*>(A.tp) + (size_t)(2 * pidx + (FWD ? 0 : 1)) * A.tws;
+}
+
 // v < 64q  ->  v mod q. The quotient estimate k = floor(t * mq / 2^24) from
 // t = floor(v / 2^(kb-8)) and mq = floor(2^(kb+16) / q) satisfies
 // v/q - 2 < k <= v/q, so v - k q lies in [0, 2q) and one subtraction ends it.
@@ -96,6 +144,37 @@ __device__ __forceinline__ u64 reduce_lazy(u64 v, u64 q, int kb, uint32_t mq) {
   return r >= q ? r - q : r;
 }
 
+// Products by halves: per-prime constants of the reductions.
+struct HalfMod {
+  u64 q, nq2;     // q, -2q mod 2^64
+  u32 n0, n1;     // -q mod 2^64
+  u32 mq, s1, s2; // floor(2^(kb+16) / q); v >> (kb - 6) as a funnel shift by s1 <= 32 and a shift by s2
+};
+__device__ __forceinline__ HalfMod half_mod(const Modulus& m) {
+  HalfMod h;
+  h.q = m.q;
+  h.nq2 = 0 - 2 * m.q;
+  h.n0 = (u32)(0 - m.q);
+  h.n1 = (u32)((0 - m.q) >> 32);
+  h.mq = (u32)(m.mu >> 47);
+  const int s = m.kbits - 6;
+  h.s1 = s < 32 ? s : 32;
+  h.s2 = s < 32 ? 0 : s - 32;
+  return h;
+}
+// v < 512q (q below 2^55)  ->  v mod q in [0, 2q): the quotient estimate
+// k = floor(t mq / 2^22) from t = floor(v / 2^(kb-6)), t mq <= (v / q) 2^22 < 2^31;
+// the truncations leave v/q - k below 1 + 2^-5 + 2^-7.
+__device__ __forceinline__ u64 reduce_half(u64 v, const HalfMod& m) {
+  const u32 lo = (u32)v, hi = (u32)(v >> 32);
+  const u32 k = ((__funnelshift_rc(lo, hi, m.s1) >> m.s2) * m.mq) >> 22;
+  u32 r0, r1;
+  asm("mad.lo.cc.u32 %0, %2, %3, %5;\n\tmadc.hi.u32 %1, %2, %3, %6;\n\tmad.lo.u32 %1, %2, %4, %1;"
+      : "=&r"(r0), "=&r"(r1)
+      : "r"(k), "r"(m.n0), "r"(m.n1), "r"(lo), "r"(hi));
+  return ((u64)r1 << 32) | r0;
+}
+
 // m = 5N/2: the four-way split of Phi_10(X^(N/4)) on four words a_j (the
 // quarters' words at one position), factored through the quadratics
 // y^2 - c y + 1 = (y - xi^e)(y - xi^-e), c = xi^e + xi^-e, e = 1 and 3. Both
@@ -104,7 +183,7 @@ __device__ __forceinline__ u64 reduce_lazy(u64 v, u64 q, int kb, uint32_t mq) {
 // quadratics share the products c_1 a3 and c_1 (a2 + a3); each remainder is
 // then evaluated at its two roots. Forward: 6 Shoup products per 4 words,
 // inputs below 4q give outputs below 16q, in the order xi^1, xi^3, xi^7, xi^9.
-// Inverse (inputs below 2q): the remainders from the root values, then
+// Inverse (inputs below off, a multiple of q with 2 off + q < 2^64): the remainders from the root values, then
 // a3 = (r0 - s0) / (1 - 2 c_1), a2 + a3 = (s1 - r1) / (1 - 2 c_1),
 // a1 = r1 - c_1 (a2 + a3), a0 = r0 + a2 + c_1 a3, scaled by 4/N: 10 products,
 // canonical. Constants per prime (value, Shoup pairs): forward c_1, xi, xi^3,
@@ -127,14 +206,14 @@ __device__ __forceinline__ void split4_fwd(u64& a0, u64& a1, u64& a2, u64& a3, c
   a2 = s0 + shoup_lazy(s1, x7.x, x7.y, q);
 }
 __device__ __forceinline__ void split4_inv(u64& b0, u64& b1, u64& b2, u64& b3, const ulonglong2* __restrict__ c,
-                                           u64 q) {
+                                           u64 q, u64 off) {
   const ulonglong2 k1 = __ldg(c + 5), x1 = __ldg(c + 6), k3 = __ldg(c + 7), x3 = __ldg(c + 8);
-  const u64 r1 = shoup(b0 - b3 + 2 * q, k1.x, k1.y, q);
+  const u64 r1 = shoup(b0 - b3 + off, k1.x, k1.y, q);
   const u64 r0 = b0 + q - shoup(r1, x1.x, x1.y, q);
-  const u64 s1 = shoup(b1 - b2 + 2 * q, k3.x, k3.y, q);
+  const u64 s1 = shoup(b1 - b2 + off, k3.x, k3.y, q);
   const u64 s0 = b1 + q - shoup(s1, x3.x, x3.y, q);
   const ulonglong2 d = __ldg(c + 9), sg = __ldg(c + 10), c1 = __ldg(c + 11);
-  const u64 a3 = shoup(r0 - s0 + 3 * q, d.x, d.y, q);
+  const u64 a3 = shoup(r0 - s0 + off + q, d.x, d.y, q);
   const u64 S = shoup(s1 - r1 + q, d.x, d.y, q);
   const u64 a2 = S >= a3 ? S - a3 : S + q - a3;
   const u64 u1 = shoup(r1, sg.x, sg.y, q), v1 = shoup(S, c1.x, c1.y, q);
@@ -304,7 +383,7 @@ __global__ void __launch_bounds__(512) k_ntt(NttArgs A, int logS, int logCPB, in
     const int n4 = W >> 2;
     for (int i = tid; i < n4; i += T) {
       u64 b0 = sm[swz(i)], b1 = sm[swz(i + n4)], b2 = sm[swz(i + 2 * n4)], b3 = sm[swz(i + 3 * n4)];
-      split4_inv(b0, b1, b2, b3, spl, q);
+      split4_inv(b0, b1, b2, b3, spl, q, 2 * q);
       sm[swz(i)] = b0;
       sm[swz(i + n4)] = b1;
       sm[swz(i + 2 * n4)] = b2;
@@ -313,7 +392,7 @@ __global__ void __launch_bounds__(512) k_ntt(NttArgs A, int logS, int logCPB, in
     __syncthreads();
   }
   u64 ni = 0, nip = 0;
-  if (LAST && !FWD) { ni = A.ninv[4 * pidx]; nip = A.ninv[4 * pidx + 1]; }
+  if (LAST && !FWD) { ni = A.ninv[6 * pidx]; nip = A.ninv[6 * pidx + 1]; }
   for (int lin = tid; lin < W; lin += T) {
     u64 v = sm[swz(lin)];
     if (LAST) {
@@ -395,14 +474,14 @@ __device__ __forceinline__ void ntt16_tile(const NttArgs& A, int logCPB, int m0,
   u64 wni = 0, wnip = 0;
   u64 cni = 0, cnip = 0;
   if (LAST && !FWD) {
-    ni = A.ninv[4 * pidx];
-    nip = A.ninv[4 * pidx + 1];
-    wni = A.ninv[4 * pidx + 2];
-    wnip = A.ninv[4 * pidx + 3];
+    const u64* nv = A.ninv + 6 * pidx;
+    ni = nv[0];
+    nip = nv[1];
+    wni = nv[2];
+    wnip = nv[3];
     if (RING == 3) {
-      const ulonglong2 c0 = __ldg(tw);
-      cni = c0.x;
-      cnip = c0.y;
+      cni = nv[4];
+      cnip = nv[5];
     }
   }
   const int kb = A.mods[pidx].kbits;
@@ -474,7 +553,7 @@ __device__ __forceinline__ void ntt16_tile(const NttArgs& A, int logCPB, int m0,
           if (jj == ns - 1) {
             const ulonglong2* spl = reinterpret_cast<const ulonglong2*>(A.split + (size_t)pidx * kSplitWords);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) split4_inv(x[k], x[k + 4], x[k + 8], x[k + 12], spl, q);
+            for (int k = 0; k < 4; ++k) split4_inv(x[k], x[k + 4], x[k + 8], x[k + 12], spl, q, q2);
           }
           continue;
         }
@@ -559,10 +638,372 @@ __device__ __forceinline__ void ntt16_tile(const NttArgs& A, int logCPB, int m0,
   }
 }
 
-template <bool FWD, bool COLS, bool LAST, int LOGS, bool SRC = false, int RING = 1>
+template <bool FWD, bool COLS, bool LAST, int LOGS, bool SRC, int RING>
 __global__ void __launch_bounds__(256, RING == 5 ? SS_NTT_MINB_R5 : (FWD ? SS_NTT_MINB_F : SS_NTT_MINB_I))
     k_ntt16(NttArgs A, int logCPB, int m0) {
   ntt16_tile<FWD, COLS, LAST, LOGS, SRC, RING>(A, logCPB, m0, blockIdx.x, blockIdx.y);
+}
+
+// ---------------------------------------------------------------- products by halves
+// Transforms of N >= 8192 on primes below 2^55 (nine spare bits in a word). With
+// a = h 2^32 + l, w_0 = w and w_1 = 2^32 w mod q, a w = l w_0 + h w_1 (mod q), a
+// sum below 2^33 q, so its quotient by 2q is one 32-bit word and the product
+// costs 26 cycles of the multiply pipe per warp (five 64-bit products at four,
+// three 32-bit ones at two) where the 64-bit Shoup product costs 32, with fewer
+// adds (half_mul; register-only loops, ncu pipe counters: forward butterflies
+// 30.2 cycles a warp against 40.8, inverse ones 30.1 against 49, which also
+// reduce every sum). A twiddle is 24 bytes (w_0, w_1, p_0, p_1).
+// Bounds. Forward: the first stage lifts its upper inputs by 128q and every
+// stage then subtracts products (below 6q, at most 16 stages) without an offset:
+// words stay below 4q + 128q + 96q. Inverse: a round starts below 32q, sums
+// double per stage (below 512q < 2^64) and differences are lifted by 32q 2^j;
+// at a round's end only the words that are sums of all its stages, or of the
+// last three, exceed 32q and are reduced.
+// One stage of half-distance step * 2^j on sixteen words of spacing `step`;
+// slot(j, blk) is the shared-memory slot of the twiddle of block blk.
+template <bool FWD, class Slot>
+__device__ __forceinline__ void half_stage(u64 (&x)[16], int j, int jj, const ulonglong2* tw, const uint2* tp,
+                                           const HalfMod& m, bool lift, Slot slot) {
+  const int d = 1 << j;
+#pragma unroll
+  for (int blk = 0; blk < 8; ++blk) {
+    if (blk < 8 / d) {
+      const int at = slot(j, blk);
+      const ulonglong2 w = tw[at];
+      const uint2 p = tp[at];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (i < d) {
+          const int k = blk * 2 * d + i;
+          u64 U = x[k];
+          const u64 V = x[k + d];
+          if (FWD) {
+            if (lift) U += m.q << 7;
+            const u64 t = half_mul(V, w.x, w.y, p.x, p.y, m.nq2);
+            x[k] = U + t;
+            x[k + d] = U - t;
+          } else {
+            x[k] = U + V;
+            x[k + d] = half_mul(U - V + (m.q << (5 + jj)), w.x, w.y, p.x, p.y, m.nq2);
+          }
+        }
+      }
+    }
+  }
+}
+// end of an inverse round of `ns` stages: back below 32q
+__device__ __forceinline__ void half_settle(u64 (&x)[16], int ns, const HalfMod& m) {
+#pragma unroll
+  for (int k = 0; k < 16; ++k)
+    if (k < (1 << (4 - ns)) || (ns == 4 && k == 1)) x[k] = reduce_half(x[k], m);
+}
+
+// Column phase: a tile is CPB = 2^CL columns (stride 2^LOG2N words) of S = 2^LOGS
+// rows of one polynomial; S CPB / 16 threads. Every address in shared and global
+// memory is a per-thread base plus a constant, and the phase's S twiddles are in
+// shared memory (6 KiB at most; copied while the words load): with runtime tile
+// shapes and twiddles from global memory the phase spent 22.4 instructions a
+// warp and butterfly where the butterfly itself takes 13.
+// The transform's top is node 1: of X^N + 1 (pre_w1, post_scale: PolySet), the
+// m = 3N split (RING 3) or, with its children, the m = 5N/2 split (RING 5).
+template <int CL>
+__device__ __forceinline__ int col_swz(int lin) {
+  // eight columns: rows 16 apart would share banks; odd groups of 16 rows swap row pairs
+  return CL == 3 ? lin ^ (((lin >> 7) & 1) << 3) : lin;
+}
+
+template <bool FWD, int LOGS, int LOG2N, int CL, int RING>
+__device__ __forceinline__ void ntt16_cols(const NttArgs& A, int tile, int poly) {
+  extern __shared__ u64 sm[];
+  constexpr int S = 1 << LOGS, G = S / 16, W = LOGS < 8 ? LOGS - 4 : 4;
+  constexpr long STRIDE = 1L << LOG2N;
+  u64* ptr;
+  int pidx;
+  if (!poly_of(A, poly, ptr, pidx)) return;
+  const int tid = threadIdx.x;
+  ulonglong2* twS = reinterpret_cast<ulonglong2*>(sm);
+  uint2* tpS = reinterpret_cast<uint2*>(twS + S);
+  u64* data = reinterpret_cast<u64*>(tpS + S);
+  {
+    const ulonglong2* gw = half_tw<FWD>(A, pidx);
+    const uint4* gp = reinterpret_cast<const uint4*>(half_tp<FWD>(A, pidx));
+    constexpr int T = S << CL >> 4;
+#pragma unroll
+    for (int i = 0; i < S; i += T)
+      if (T <= S || tid < S) cp16(twS + i + tid, gw + i + tid);
+#pragma unroll
+    for (int i = 0; i < S / 2; i += T)
+      if (T <= S / 2 || tid < S / 2) cp16(reinterpret_cast<uint4*>(tpS) + i + tid, gp + i + tid);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  }
+  const int c = tid & ((1 << CL) - 1), rest = tid >> CL;
+  u64* col = ptr + ((long)tile << CL) + c;
+  const HalfMod hm = half_mod(A.mods[pidx]);
+  const u64 q = hm.q;
+  u64 x[16];
+  // wide round: rows rest + G k; narrow round: rows 16 rest + k
+#pragma unroll
+  for (int k = 0; k < 16; ++k) x[k] = FWD ? col[(rest + (long)G * k) * STRIDE] : col[(16 * rest + (long)k) * STRIDE];
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  __syncthreads();
+  auto wide_slot = [](int j, int blk) { return tw_slot((1 << (3 - j)) + blk, LOGS - 4 + j, W); };
+  auto narrow_slot = [rest](int j, int blk) { return (1 << (LOGS - 1 - j)) + (blk << W) + rest; };
+  const ulonglong2* spl =
+      RING == 5 ? reinterpret_cast<const ulonglong2*>(A.split + (size_t)pidx * kSplitWords) : nullptr;
+  if (FWD) {
+    int j0 = 3;
+    if (RING == 5) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) split4_fwd(x[k], x[k + 4], x[k + 8], x[k + 12], spl, q);
+      j0 = 1;
+    } else if (RING == 3) {
+      const ulonglong2 w = twS[1];
+      const uint2 p = tpS[1];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const u64 U = x[k] + (q << 7), V = x[k + 8];
+        const u64 t = half_mul(V, w.x, w.y, p.x, p.y, hm.nq2);
+        x[k] = U + t;
+        x[k + 8] = U + V - t;
+      }
+      j0 = 2;
+    } else if (A.pre_w1) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const u64 U = x[k] + (q << 7), V = x[k + 8];  // V < 4q
+        x[k] = U + V;
+        x[k + 8] = U - V;
+      }
+      j0 = 2;
+    }
+#pragma unroll
+    for (int j = 3; j >= 0; --j)
+      if (j <= j0) half_stage<true>(x, j, 0, twS, tpS, hm, RING == 5 ? j == 1 : RING == 1 && j == 3, wide_slot);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) data[col_swz<CL>(((rest + G * k) << CL) + c)] = x[k];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) x[k] = data[col_swz<CL>(((16 * rest + k) << CL) + c)];
+#pragma unroll
+    for (int j = LOGS - 5; j >= 0; --j) half_stage<true>(x, j, 0, twS, tpS, hm, false, narrow_slot);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) col[(16 * rest + (long)k) * STRIDE] = x[k];
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) half_stage<false>(x, j, j, twS, tpS, hm, false, narrow_slot);
+  half_settle(x, 4, hm);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) data[col_swz<CL>(((16 * rest + k) << CL) + c)] = x[k];
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 16; ++k) x[k] = data[col_swz<CL>(((rest + G * k) << CL) + c)];
+  constexpr int NS = LOGS - 4;  // stages j = 4 - NS .. 3, the last one (or two) with N^-1
+  constexpr int JE = RING == 5 ? 2 : 3;
+  if constexpr (4 - NS < JE) {
+#pragma unroll
+    for (int j = 4 - NS; j < JE; ++j) half_stage<false>(x, j, j - (4 - NS), twS, tpS, hm, false, wide_slot);
+  }
+  const u64* nv = A.ninv + 6 * pidx;
+  const u64 off = q << (5 + NS - 1);  // above every input of the last stage
+  if (RING == 5) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) split4_inv(x[k], x[k + 4], x[k + 8], x[k + 12], spl, q, off);
+  } else if (RING == 3) {
+    const u64 ni = nv[0], nip = nv[1], w = nv[2], wp = nv[3], cn = nv[4], cnp = nv[5];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const u64 sv = x[k] + x[k + 8], dv = x[k] - x[k + 8] + off;
+      const u64 lo = shoup(sv, ni, nip, q), cr = shoup(dv, cn, cnp, q);
+      x[k] = lo >= cr ? lo - cr : lo + q - cr;
+      x[k + 8] = shoup(dv, w, wp, q);
+    }
+  } else if (A.post_scale) {  // N^-1 and N^-1 psi^(-N/2) left to the consumer
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const u64 U = x[k], V = x[k + 8];
+      x[k] = U + V;
+      x[k + 8] = U - V + off;
+    }
+  } else {
+    const u64 ni = nv[0], nip = nv[1], w = nv[2], wp = nv[3];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const u64 U = x[k], V = x[k + 8];
+      x[k] = shoup(U + V, ni, nip, q);
+      x[k + 8] = shoup(U - V + off, w, wp, q);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 16; ++k) col[(rest + (long)G * k) * STRIDE] = x[k];
+}
+
+constexpr int kColTile = 11;  // log2 words of a column tile: 128 threads
+template <int LOGS, int CL>
+constexpr size_t col_smem() {
+  return ((size_t)24 << LOGS) + ((size_t)8 << (LOGS + CL));
+}
+
+template <bool FWD, int LOGS, int LOG2N, int CL, int RING>
+__global__ void __launch_bounds__(128, FWD ? SS_COLS_F : SS_COLS_I) k_ntt16_cols(NttArgs A) {
+  ntt16_cols<FWD, LOGS, LOG2N, CL, RING>(A, blockIdx.x, blockIdx.y);
+}
+
+// Chunk phase: a row is one chunk (S = 2^LOGS words) of one polynomial; S / 16 threads (16 or
+// 8, within one warp) hold it, sixteen words each, so its two register rounds
+// exchange words through the warp's own shared memory with warp barriers only.
+// A CTA takes the same chunks of several polynomials of one limb: NP = 2^lnp of
+// them times NC = rows / NP chunks. Their twiddles, 24 bytes a node, are copied
+// to shared memory once per CTA (cp.async, while the first words load), where
+// one polynomial's chunks per CTA read each node from L2 once per polynomial
+// with its latency exposed in every stage (forward chunk phase, 328 limbs of
+// 2^16 words, products by halves: 129 us, the multiply pipe 60 % busy).
+// Polynomials that the set skips (a ModUp digit's own limbs) are left out of the
+// groups: the v-th polynomial of a limb is the v-th that is transformed.
+// word r of a row: pairs of words stay adjacent (16-byte accesses); the pairs of
+// a group of 16 are permuted by the group's index, so eight threads that each
+// read a pair of their own group, and sixteen that read one word each of one
+// group, touch all banks once
+__device__ __forceinline__ int row_swz(int r) { return r ^ (((r >> 4) & 7) << 1); }
+
+struct RowPlan {
+  int lnp, groups;  // log2 NP, groups of NP polynomials per limb (at most)
+};
+
+template <bool FWD, int LOGS, bool SRC>
+__device__ __forceinline__ void ntt16_rows(const NttArgs& A, const RowPlan& R, int item, int limb) {
+  extern __shared__ u64 sm[];
+  constexpr int S = 1 << LOGS, TPR = S / 16, LT = LOGS - 4;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int lnc = (31 - __clz(blockDim.x)) - LT - R.lnp;  // log2 NC
+  const int group = item % R.groups, cg = item / R.groups;
+  // the limb's polynomials: all, or those whose digit is not the limb's own
+  const bool own = A.skip_w > 0 && limb < A.nq && limb < A.skip_level;
+  const int per = own ? A.skip_mod - 1 : A.n_outer;
+  const int nv = own ? (A.n_outer / A.skip_mod) * per : A.n_outer;
+  const int v0 = group << R.lnp;
+  if (v0 >= nv) return;
+  const int pidx = limb < A.nq ? A.q0 + limb : A.L + (limb - A.nq);
+  const int n1 = A.N >> LOGS;
+  // twiddles of the CTA's chunks
+  ulonglong2* twS = reinterpret_cast<ulonglong2*>(sm);
+  uint2* tpS = reinterpret_cast<uint2*>(twS + (S << lnc));
+  u64* data = reinterpret_cast<u64*>(tpS + (S << lnc)) + (size_t)(tid >> 5) * 512;
+  {
+    const size_t at = (size_t)n1 + ((size_t)cg << (lnc + LOGS));
+    const ulonglong2* gw = half_tw<FWD>(A, pidx) + at;
+    const uint4* gp = reinterpret_cast<const uint4*>(half_tp<FWD>(A, pidx) + at);
+    for (int i = tid; i < (S << lnc); i += blockDim.x) cp16(twS + i, gw + i);
+    for (int i = tid; i < (S << lnc) / 2; i += blockDim.x) cp16(reinterpret_cast<uint4*>(tpS) + i, gp + i);
+  }
+  const int row = tid >> LT, lr = tid & (TPR - 1);
+  const int v = v0 + (row & ((1 << R.lnp) - 1));
+  const int chl = row >> R.lnp;
+  const bool valid = v < nv;
+  long off = 0, soff = 0;
+  if (valid) {
+    int o = v;
+    if (own) {
+      const int b = v / per, jj = v - b * per;
+      o = b * A.skip_mod + jj + (jj >= limb / A.skip_w ? 1 : 0);
+    }
+    const long in_poly = (long)limb * A.N + ((long)((cg << lnc) + chl) << LOGS);
+    off = (long)o * A.outer_stride + in_poly;
+    soff = SRC ? (long)o * A.src_os + in_poly : off;
+  }
+  const u64* src = (SRC ? A.src : A.base) + soff;
+  u64* dst = A.base + off;
+  const HalfMod hm = half_mod(A.mods[pidx]);
+  const u64 q = hm.q;
+  u64* mine = data + (lane >> LT) * S;  // this thread's row in the warp's shared memory
+  u64 x[16];
+  // this warp's rows in linear order: lane l moves the pairs l, l + 32, ... of each
+  constexpr int RPW = 32 / TPR;  // rows per warp
+  if (FWD) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) x[k] = valid ? src[lr + TPR * k] : 0;
+  } else {
+#pragma unroll
+    for (int rw = 0; rw < RPW; ++rw) {
+      const u64* rp = reinterpret_cast<const u64*>(__shfl_sync(0xffffffffu, (unsigned long long)src, rw * TPR));
+      const bool ok = __shfl_sync(0xffffffffu, valid ? 1 : 0, rw * TPR) != 0;
+#pragma unroll
+      for (int i = 0; i < S / 64; ++i) {
+        const int r = 2 * (lane + 32 * i);
+        if (ok) cp16(data + rw * S + row_swz(r), rp + r);
+      }
+    }
+  }
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  __syncthreads();
+  if (!__any_sync(0xffffffffu, valid)) return;
+  const ulonglong2* tw = twS + chl * S;
+  const uint2* tp = tpS + chl * S;
+  // the narrow round holds words 16 lr .. 16 lr + 15, the wide round words lr + TPR k
+  auto wide_slot = [](int j, int blk) { return (1 << (3 - j)) + blk; };
+  auto narrow_slot = [lr](int j, int blk) { return (1 << (LOGS - 1 - j)) + (blk << LT) + lr; };
+  auto put_own = [&] {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      *reinterpret_cast<ulonglong2*>(mine + row_swz(16 * lr + 2 * i)) = make_ulonglong2(x[2 * i], x[2 * i + 1]);
+  };
+  auto get_own = [&] {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(mine + row_swz(16 * lr + 2 * i));
+      x[2 * i] = t.x;
+      x[2 * i + 1] = t.y;
+    }
+  };
+  if (FWD) {
+#pragma unroll
+    for (int j = 3; j >= 0; --j) half_stage<true>(x, j, 0, tw, tp, hm, false, wide_slot);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) mine[row_swz(lr + TPR * k)] = x[k];
+    __syncwarp();
+    get_own();
+#pragma unroll
+    for (int j = LOGS - 5; j >= 0; --j) half_stage<true>(x, j, 0, tw, tp, hm, false, narrow_slot);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const u64 r = reduce_half(x[k], hm), d = r - q;  // d wraps above r when r < q
+      x[k] = r < d ? r : d;
+    }
+    put_own();
+    __syncwarp();
+#pragma unroll
+    for (int rw = 0; rw < RPW; ++rw) {
+      u64* rp = reinterpret_cast<u64*>(__shfl_sync(0xffffffffu, (unsigned long long)dst, rw * TPR));
+      const bool ok = __shfl_sync(0xffffffffu, valid ? 1 : 0, rw * TPR) != 0;
+#pragma unroll
+      for (int i = 0; i < S / 64; ++i) {
+        const int r = 2 * (lane + 32 * i);
+        if (ok) *reinterpret_cast<ulonglong2*>(rp + r) = *reinterpret_cast<const ulonglong2*>(data + rw * S + row_swz(r));
+      }
+    }
+  } else {
+    get_own();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) half_stage<false>(x, j, j, tw, tp, hm, false, narrow_slot);
+    half_settle(x, 4, hm);
+    put_own();
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) x[k] = mine[row_swz(lr + TPR * k)];
+    constexpr int NS = LOGS - 4;  // stages of the wide round: half-distances 16 .. S/2
+#pragma unroll
+    for (int j = 4 - NS; j < 4; ++j) half_stage<false>(x, j, j - (4 - NS), tw, tp, hm, false, wide_slot);
+    half_settle(x, NS, hm);
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      if (valid) dst[lr + TPR * k] = x[k];
+  }
+}
+
+template <bool FWD, int LOGS, bool SRC>
+__global__ void __launch_bounds__(128, FWD ? SS_ROWS_F : SS_ROWS_I) k_ntt16_rows(NttArgs A, RowPlan R) {
+  ntt16_rows<FWD, LOGS, SRC>(A, R, blockIdx.x, blockIdx.y);
 }
 
 // ---------------------------------------------------------------- persistent multi-transform phase
@@ -577,7 +1018,8 @@ __global__ void __launch_bounds__(256, RING == 5 ? SS_NTT_MINB_R5 : (FWD ? SS_NT
 constexpr int kMaxNttJobs = 24;
 struct NttJob {
   NttArgs A;
-  int logS, logCPB, m0, tiles, start;
+  int logS, log2n, tiles, start;  // log2 column and chunk length; tiles per polynomial (columns) or limb (chunks)
+  RowPlan rows;  // chunk phase
   int ring;  // the context's m_odd: 3 (m = 3N) or 5 (m = 5N/2) give the column phase its split; 1 none
 };
 struct NttMulti {
@@ -586,14 +1028,17 @@ struct NttMulti {
 };
 
 // a separate function per instantiation, so each keeps its own register allocation
-template <bool FWD, bool COLS, bool LAST, int LOGS, bool SRC, int RING = 1>
-__device__ __noinline__ void ntt16_tile_fn(const NttArgs& A, int logCPB, int m0, int tile, int poly) {
-  ntt16_tile<FWD, COLS, LAST, LOGS, SRC, RING>(A, logCPB, m0, tile, poly);
+template <bool FWD, int LOGS, int LOG2N, int RING>
+__device__ __noinline__ void ntt16_cols_fn(const NttArgs& A, int tile, int poly) {
+  ntt16_cols<FWD, LOGS, LOG2N, kColTile - LOGS, RING>(A, tile, poly);
+}
+template <bool FWD, int LOGS, bool SRC>
+__device__ __noinline__ void ntt16_rows_fn(const NttArgs& A, const RowPlan& R, int item, int limb) {
+  ntt16_rows<FWD, LOGS, SRC>(A, R, item, limb);
 }
 
-template <bool FWD, bool COLS, bool LAST, bool SRC>
-__global__ void __launch_bounds__(256, FWD ? SS_NTT_MINB_F : SS_NTT_MINB_I)
-    k_ntt16_multi(const __grid_constant__ NttMulti M) {
+template <bool FWD, bool COLS, bool SRC>
+__global__ void __launch_bounds__(128, 6) k_ntt16_multi(const __grid_constant__ NttMulti M) {
   for (int t = blockIdx.x; t < M.total; t += gridDim.x) {
     int j = 0;
     while (j + 1 < M.njobs && t >= M.j[j + 1].start) ++j;
@@ -601,44 +1046,104 @@ __global__ void __launch_bounds__(256, FWD ? SS_NTT_MINB_F : SS_NTT_MINB_I)
     const int local = t - J.start;
     const int poly = local / J.tiles, tile = local - poly * J.tiles;
     if constexpr (COLS) {
-      if (J.ring == 3 || J.ring == 5) {
-        if (J.ring == 3) {
-          switch (J.logS) {
-            case 5: ntt16_tile_fn<FWD, COLS, LAST, 5, SRC, 3>(J.A, J.logCPB, J.m0, tile, poly); break;
-            case 6: ntt16_tile_fn<FWD, COLS, LAST, 6, SRC, 3>(J.A, J.logCPB, J.m0, tile, poly); break;
-            case 7: ntt16_tile_fn<FWD, COLS, LAST, 7, SRC, 3>(J.A, J.logCPB, J.m0, tile, poly); break;
-            default: ntt16_tile_fn<FWD, COLS, LAST, 8, SRC, 3>(J.A, J.logCPB, J.m0, tile, poly); break;
-          }
-        } else {
-          switch (J.logS) {
-            case 6: ntt16_tile_fn<FWD, COLS, LAST, 6, SRC, 5>(J.A, J.logCPB, J.m0, tile, poly); break;
-            case 7: ntt16_tile_fn<FWD, COLS, LAST, 7, SRC, 5>(J.A, J.logCPB, J.m0, tile, poly); break;
-            default: ntt16_tile_fn<FWD, COLS, LAST, 8, SRC, 5>(J.A, J.logCPB, J.m0, tile, poly); break;
-          }
-        }
-        __syncthreads();
-        continue;
+      switch (J.ring * 16 + J.logS) {
+        case 16 + 5: ntt16_cols_fn<FWD, 5, 8, 1>(J.A, tile, poly); break;
+        case 16 + 6: ntt16_cols_fn<FWD, 6, 8, 1>(J.A, tile, poly); break;
+        case 16 + 7: ntt16_cols_fn<FWD, 7, 8, 1>(J.A, tile, poly); break;
+        case 16 + 8: ntt16_cols_fn<FWD, 8, 8, 1>(J.A, tile, poly); break;
+        case 48 + 5: ntt16_cols_fn<FWD, 5, 8, 3>(J.A, tile, poly); break;
+        case 48 + 6: ntt16_cols_fn<FWD, 6, 8, 3>(J.A, tile, poly); break;
+        case 48 + 7: ntt16_cols_fn<FWD, 7, 8, 3>(J.A, tile, poly); break;
+        case 48 + 8: ntt16_cols_fn<FWD, 8, 8, 3>(J.A, tile, poly); break;
+        case 80 + 6:
+          if (J.log2n == 7) ntt16_cols_fn<FWD, 6, 7, 5>(J.A, tile, poly);
+          else ntt16_cols_fn<FWD, 6, 8, 5>(J.A, tile, poly);
+          break;
+        case 80 + 7: ntt16_cols_fn<FWD, 7, 8, 5>(J.A, tile, poly); break;
+        default: ntt16_cols_fn<FWD, 8, 8, 5>(J.A, tile, poly); break;
       }
-    }
-    switch (J.logS) {
-      case 5: ntt16_tile_fn<FWD, COLS, LAST, 5, SRC>(J.A, J.logCPB, J.m0, tile, poly); break;
-      case 6: ntt16_tile_fn<FWD, COLS, LAST, 6, SRC>(J.A, J.logCPB, J.m0, tile, poly); break;
-      case 7: ntt16_tile_fn<FWD, COLS, LAST, 7, SRC>(J.A, J.logCPB, J.m0, tile, poly); break;
-      default: ntt16_tile_fn<FWD, COLS, LAST, 8, SRC>(J.A, J.logCPB, J.m0, tile, poly); break;
+    } else if (J.log2n == 7) {
+      ntt16_rows_fn<FWD, 7, SRC>(J.A, J.rows, tile, poly);  // poly counts limbs here
+    } else {
+      ntt16_rows_fn<FWD, 8, SRC>(J.A, J.rows, tile, poly);
     }
     __syncthreads();  // the next tile reuses the shared memory
   }
 }
 
-template <bool FWD, bool COLS, bool LAST, bool SRC = false, int RING = 1>
-void launch16(int logS, dim3 g, int thr, size_t smem, cudaStream_t st, const NttArgs& A, int logc, int m0) {
-  switch (logS) {
-    case 5: k_ntt16<FWD, COLS, LAST, 5, SRC, RING><<<g, thr, smem, st>>>(A, logc, m0); break;
-    case 6: k_ntt16<FWD, COLS, LAST, 6, SRC, RING><<<g, thr, smem, st>>>(A, logc, m0); break;
-    case 7: k_ntt16<FWD, COLS, LAST, 7, SRC, RING><<<g, thr, smem, st>>>(A, logc, m0); break;
-    default: k_ntt16<FWD, COLS, LAST, 8, SRC, RING><<<g, thr, smem, st>>>(A, logc, m0); break;
+// column phase of one transform by halves
+template <bool FWD, int LOGS, int LOG2N, int RING>
+void launch_cols_as(int npoly, cudaStream_t st, const NttArgs& A) {
+  constexpr int CL = kColTile - LOGS;
+  k_ntt16_cols<FWD, LOGS, LOG2N, CL, RING><<<dim3(1 << (LOG2N - CL), npoly), 128, col_smem<LOGS, CL>(), st>>>(A);
+}
+template <bool FWD>
+void launch_cols(int ring, int logS, int log2n, int npoly, cudaStream_t st, const NttArgs& A) {
+  switch (ring * 16 + logS) {
+    case 16 + 5: launch_cols_as<FWD, 5, 8, 1>(npoly, st, A); break;
+    case 16 + 6: launch_cols_as<FWD, 6, 8, 1>(npoly, st, A); break;
+    case 16 + 7: launch_cols_as<FWD, 7, 8, 1>(npoly, st, A); break;
+    case 16 + 8: launch_cols_as<FWD, 8, 8, 1>(npoly, st, A); break;
+    case 48 + 5: launch_cols_as<FWD, 5, 8, 3>(npoly, st, A); break;
+    case 48 + 6: launch_cols_as<FWD, 6, 8, 3>(npoly, st, A); break;
+    case 48 + 7: launch_cols_as<FWD, 7, 8, 3>(npoly, st, A); break;
+    case 48 + 8: launch_cols_as<FWD, 8, 8, 3>(npoly, st, A); break;
+    case 80 + 6:
+      if (log2n == 7) launch_cols_as<FWD, 6, 7, 5>(npoly, st, A);
+      else launch_cols_as<FWD, 6, 8, 5>(npoly, st, A);
+      break;
+    case 80 + 7: launch_cols_as<FWD, 7, 8, 5>(npoly, st, A); break;
+    default: launch_cols_as<FWD, 8, 8, 5>(npoly, st, A); break;
   }
 }
+
+// one phase of a transform in the Shoup form
+template <bool FWD, bool COLS, bool LAST, bool SRC = false, int RING = 1>
+void launch16(int logS, dim3 g, int thr, size_t smem, cudaStream_t st, const NttArgs& A, int logc, int m0) {
+  if constexpr (COLS) {
+    switch (logS) {
+      case 5: k_ntt16<FWD, COLS, LAST, 5, SRC, RING><<<g, thr, smem, st>>>(A, logc, m0); return;
+      case 6: k_ntt16<FWD, COLS, LAST, 6, SRC, RING><<<g, thr, smem, st>>>(A, logc, m0); return;
+      default: break;
+    }
+  }
+  if (logS == 7) k_ntt16<FWD, COLS, LAST, 7, SRC, RING><<<g, thr, smem, st>>>(A, logc, m0);
+  else k_ntt16<FWD, COLS, LAST, 8, SRC, RING><<<g, thr, smem, st>>>(A, logc, m0);
+}
+
+// How one launch of the chunk phase covers a set: the polynomials of a limb in
+// groups of up to a CTA's rows (fewer when the limb has fewer), and the shared
+// memory a CTA needs.
+RowPlan row_plan(const PolySet& s, int rows) {
+  RowPlan R;
+  R.lnp = 0;
+  while ((1 << R.lnp) < rows && (1 << R.lnp) < s.n_outer) ++R.lnp;
+  R.groups = (s.n_outer + (1 << R.lnp) - 1) >> R.lnp;
+  return R;
+}
+size_t row_smem(int logS, int thr, int lnp) {
+  const int rows = thr >> (logS - 4);
+  return ((size_t)(rows >> lnp) << logS) * 24 + (size_t)rows * 8 * (1 << logS);
+}
+
+template <bool FWD, bool SRC>
+void launch_rows(int logS, const PolySet& s, cudaStream_t st, const NttArgs& A) {
+  int thr = 128;
+  RowPlan R = row_plan(s, thr >> (logS - 4));
+  while (row_smem(logS, thr, R.lnp) > 48 * 1024) {  // few polynomials: fewer rows, not more than the default limit
+    thr /= 2;
+    R = row_plan(s, thr >> (logS - 4));
+  }
+  const dim3 g(((A.N >> logS) / ((thr >> (logS - 4)) >> R.lnp)) * R.groups, s.nl);
+  const size_t smem = row_smem(logS, thr, R.lnp);
+  if (logS == 7) k_ntt16_rows<FWD, 7, SRC><<<g, thr, smem, st>>>(A, R);
+  else k_ntt16_rows<FWD, 8, SRC><<<g, thr, smem, st>>>(A, R);
+}
+
+// log2 of the chunk length N2 of the two-phase split: 256, except that the
+// m = 5N/2 ring needs at least 64 column words (its inverse split takes the
+// column phase's last two stages in one register round)
+int chunk_log(const Context& C) { return C.m_odd == 5 && C.logN - 8 < 6 ? C.logN - 6 : 8; }
 
 NttArgs make_args(Context& C, const PolySet& s) {
   NttArgs A;
@@ -655,6 +1160,8 @@ NttArgs make_args(Context& C, const PolySet& s) {
   A.skip_level = s.skip_level;
   A.mods = reinterpret_cast<const Modulus*>(C.d_mod);
   A.tw = C.d_tw;
+  A.tp = C.d_tp;
+  A.tws = C.N + (C.N >> chunk_log(C));
   A.ninv = C.d_ninv;
   A.split = C.d_split;
   A.src = nullptr;
@@ -697,17 +1204,24 @@ NttMerger*& ntt_merger() {
   return m;
 }
 
-// log2 of the chunk length N2 of the two-phase split: 256, except that the
-// m = 5N/2 ring needs at least 64 column words (its inverse split takes the
-// column phase's last two stages in one register round)
-static int chunk_log(const Context& C) { return C.m_odd == 5 && C.logN - 8 < 6 ? C.logN - 6 : 8; }
+// Products by halves: slot of node k in one prime's and direction's table of
+// N + N1 slots (see half_tw).
+int ntt_tw_slots(const Context& C) { return C.N + (C.N >> chunk_log(C)); }
+int ntt_tw_slot(const Context& C, int k) {
+  const int l2 = chunk_log(C), l1 = C.logN - l2;
+  int depth = 0;
+  while ((2 << depth) <= k) ++depth;
+  if (depth < l1) return tw_slot(k, l1 - 1 - depth, l1 < 8 ? l1 - 4 : 4);  // the column phase's stages come first
+  const int s = depth - l1, chunk = (k >> s) - (1 << l1), local = (1 << s) + (k & ((1 << s) - 1));
+  return (1 << l1) + (chunk << l2) + tw_slot(local, l2 - 1 - s, l2 - 4);
+}
 
 // src: optional out-of-place source read by the first phase (inverse only)
 static void launch(Context& C, const PolySet& s, bool fwd, cudaStream_t st, const u64* src = nullptr,
                    long src_os = 0) {
   int npoly = s.n_outer * s.nl;
   if (npoly == 0) return;
-  if (ntt_merger() && C.N > TILE && !is_dry(C)) {
+  if (ntt_merger() && C.N > TILE && C.d_tp && !is_dry(C)) {
     ntt_merger()->submit(NttReq{&C, s, src, src_os}, fwd, st);
     return;
   }
@@ -742,7 +1256,21 @@ static void launch(Context& C, const PolySet& s, bool fwd, cudaStream_t st, cons
     const int logc1 = tl - log1, logc2 = tl - log2n;
     dim3 g1(1 << (log2n - logc1), npoly), g2(1 << (log1 - logc2), npoly);
     const int thr = tile / 16;
-    if (fwd) {
+    if (A.tp) {
+      NttArgs A1 = A;
+      if (src) {
+        A1.src = src;
+        A1.src_os = src_os;
+      }
+      if (fwd) {
+        launch_cols<true>(C.m_odd, log1, log2n, npoly, st, A);
+        launch_rows<true, false>(log2n, s, st, A);
+      } else {
+        if (src) launch_rows<false, true>(log2n, s, st, A1);
+        else launch_rows<false, false>(log2n, s, st, A);
+        launch_cols<false>(C.m_odd, log1, log2n, npoly, st, A);
+      }
+    } else if (fwd) {
       if (C.m_odd == 3) launch16<true, true, false, false, 3>(log1, g1, thr, smem(tile), st, A, logc1, 1);
       else if (C.m_odd == 5) launch16<true, true, false, false, 5>(log1, g1, thr, smem(tile), st, A, logc1, 1);
       else launch16<true, true, false>(log1, g1, thr, smem(tile), st, A, logc1, 1);
@@ -774,23 +1302,34 @@ static int resident_ctas() {
     int dev = 0, sms = 0;
     SS_CUDA(cudaGetDevice(&dev));
     SS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    v = sms * SS_NTT_MINB_F;
+    v = sms * 6;
     n.store(v);
   }
   return v;
 }
 
-template <bool FWD, bool COLS, bool LAST, bool SRC>
+template <bool FWD, bool COLS, bool SRC>
 static void launch_multi(const NttMulti& M, int thr, size_t smem, cudaStream_t st) {
   if (M.total == 0) return;
   const int grid = std::min(M.total, resident_ctas());
-  k_ntt16_multi<FWD, COLS, LAST, SRC><<<grid, thr, smem, st>>>(M);
+  if (smem > 48 * 1024) {  // many chunks of few polynomials: opt in once per kernel and device
+    static std::atomic<unsigned long long> done{0};
+    int dev = 0;
+    SS_CUDA(cudaGetDevice(&dev));
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(done.load() & bit)) {
+      SS_CUDA(cudaFuncSetAttribute(k_ntt16_multi<FWD, COLS, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   128 * 1024));
+      done.fetch_or(bit);
+    }
+  }
+  k_ntt16_multi<FWD, COLS, SRC><<<grid, thr, smem, st>>>(M);
   SS_CUDA(cudaGetLastError());
 }
 
-void ntt_multi(const std::vector<NttReq>& reqs, bool fwd, int tile_log, cudaStream_t st) {
-  const int tl = tile_log == 11 ? 11 : 12, tile = 1 << tl, thr = tile / 16;
-  const size_t smem = (size_t)(tile + tile / 8) * 8;
+void ntt_multi(const std::vector<NttReq>& reqs, bool fwd, cudaStream_t st) {
+  const int thr = 128;
+  const size_t smem_cols = col_smem<8, kColTile - 8>();  // the longest columns' twiddles and a tile
   for (size_t b0 = 0; b0 < reqs.size(); b0 += kMaxNttJobs) {
     const size_t b1 = std::min(reqs.size(), b0 + kMaxNttJobs);
     // phase 1 (columns forward, chunks inverse) and phase 2 of every job
@@ -798,16 +1337,20 @@ void ntt_multi(const std::vector<NttReq>& reqs, bool fwd, int tile_log, cudaStre
     P1.njobs = P2.njobs = 0;
     P1.total = P2.total = 0;
     double bytes = 0, prods = 0;
+    size_t smem_rows = 0;
     for (size_t r = b0; r < b1; ++r) {
       const NttReq& q = reqs[r];
       Context& C = *q.C;
-      if (C.N < 8192) throw Error(SS_ERR_PARAM, "merged transforms need N >= 8192");
+      if (C.N < 8192 || !C.d_tp) throw Error(SS_ERR_PARAM, "merged transforms need N >= 8192 and primes below 2^55");
       const int npoly = q.s.n_outer * q.s.nl;
       if (npoly == 0) continue;
       NttArgs A = make_args(C, q.s);
-      const int l2 = chunk_log(C), log1 = C.logN - l2, logc1 = tl - log1, logc2 = tl - l2;
-      NttJob cols{A, log1, logc1, 1, 1 << (l2 - logc1), 0, C.m_odd};
-      NttJob chunks{A, l2, logc2, 1 << log1, 1 << (log1 - logc2), 0, 1};
+      const int l2 = chunk_log(C), log1 = C.logN - l2;
+      const RowPlan R = row_plan(q.s, thr >> (l2 - 4));
+      const int rows = thr >> (l2 - 4);
+      NttJob cols{A, log1, l2, 1 << (l2 - (kColTile - log1)), 0, R, C.m_odd};
+      NttJob chunks{A, log1, l2, ((1 << log1) / (rows >> R.lnp)) * R.groups, 0, R, 1};
+      smem_rows = std::max(smem_rows, row_smem(l2, thr, R.lnp));
       if (!fwd) {  // the chunk phase reads the source (the polynomials themselves when in place)
         chunks.A.src = q.src ? q.src : q.s.base;
         chunks.A.src_os = q.src ? q.src_os : q.s.outer_stride;
@@ -818,8 +1361,8 @@ void ntt_multi(const std::vector<NttReq>& reqs, bool fwd, int tile_log, cudaStre
       j2 = fwd ? chunks : cols;
       j1.start = P1.total;
       j2.start = P2.total;
-      P1.total += npoly * j1.tiles;
-      P2.total += npoly * j2.tiles;
+      P1.total += (fwd ? npoly : q.s.nl) * j1.tiles;
+      P2.total += (fwd ? q.s.nl : npoly) * j2.tiles;
       bytes += 16.0 * C.N * active_polys(q.s);
       prods += ntt_products(C, q.s, fwd);
     }
@@ -827,11 +1370,11 @@ void ntt_multi(const std::vector<NttReq>& reqs, bool fwd, int tile_log, cudaStre
     Context& C0 = *reqs[b0].C;
     int kr = kt_begin(C0, st);
     if (fwd) {
-      launch_multi<true, true, false, false>(P1, thr, smem, st);
-      launch_multi<true, false, true, false>(P2, thr, smem, st);
+      launch_multi<true, true, false>(P1, 128, smem_cols, st);
+      launch_multi<true, false, false>(P2, thr, smem_rows, st);
     } else {
-      launch_multi<false, false, false, true>(P1, thr, smem, st);
-      launch_multi<false, true, true, false>(P2, thr, smem, st);
+      launch_multi<false, false, true>(P1, thr, smem_rows, st);
+      launch_multi<false, true, false>(P2, 128, smem_cols, st);
     }
     C0.launches += 2;
     if (kr >= 0) C0.kt.ntt_products += prods;

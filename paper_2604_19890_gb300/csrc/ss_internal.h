@@ -132,10 +132,14 @@ struct Context {
 
   // device tables
   ModDesc* d_mod = nullptr;           // [ntot]
-  u64* d_tw = nullptr;                // per prime 4N words: (psi_brv, shoup) pairs, then (psiinv_brv, shoup) pairs
+  u64* d_tw = nullptr;                // per prime 4N words: forward (w, shoup) pairs, then inverse ones; products by
+                                      //   halves: per prime and direction ntt_tw_slots pairs (w, 2^32 w mod q)
+  u32* d_tp = nullptr;                // products by halves (N >= 8192, primes below 2^55): for each pair of d_tw the
+                                      //   two half-quotients floor(w 2^31 / q); else null
   u64* d_r64 = nullptr;               // [ntot][4] 2^64 mod q; X^N + 1: 2^64 psi^(N/2) (forward node 1),
                                       //   2^64 N^-1, 2^64 N^-1 psi^(-N/2) (the inverse's last stage)
-  u64* d_ninv = nullptr;              // [ntot][4] N^{-1}, shoup, N^{-1} psi^{-N/2} (m = 3N: 2 N^{-1}), shoup
+  u64* d_ninv = nullptr;              // [ntot][6] N^{-1}, shoup, N^{-1} psi^{-N/2} (m = 3N: 2 c), shoup, (m = 3N: c =
+                                      //   (2 rho - 1)^{-1} N^{-1}), shoup
   u64* d_split = nullptr;             // m = 5N/2: [ntot][12][2] four-way split constants (forward 5, inverse 7)
   u64* d_pinv = nullptr;              // [ntot][2] p^{-1}, shoup
   u64* d_tmod = nullptr;              // [r+1][ntot][2]: p^e mod q, shoup
@@ -205,6 +209,10 @@ struct PolySet {
   bool pre_w1 = false;
   bool post_scale = false;
 };
+// Products by halves: slots per prime and direction of the twiddle tables, and
+// the slot of node k of the transform tree.
+int ntt_tw_slots(const Context& C);
+int ntt_tw_slot(const Context& C, int k);
 void ntt_forward(Context& C, const PolySet& s, cudaStream_t st);
 void ntt_inverse(Context& C, const PolySet& s, cudaStream_t st);
 // Inverse transform of the polynomials at src (same shape as s, outer stride
@@ -218,7 +226,7 @@ struct NttReq {
   const u64* src;  // out-of-place source of an inverse transform, or null
   long src_os;
 };
-void ntt_multi(const std::vector<NttReq>& reqs, bool fwd, int tile_log, cudaStream_t st);
+void ntt_multi(const std::vector<NttReq>& reqs, bool fwd, cudaStream_t st);
 // Collects the transforms that several cooperating host threads issue (the
 // batched form's lanes) and launches them merged. While a thread's hook is
 // set, its transforms of rings N >= 8192 go to submit(), which returns once

@@ -1,0 +1,73 @@
+"""Transforms that multiply by halves (N >= 8192, primes below 2^55) against the
+CPU reference, at the sizes where their tiling can go wrong: the fewest and
+ragged counts of polynomials per limb, the smallest column and chunk lengths,
+the widest primes that take this form and the first that do not, and the inputs
+that grow the lazy words most. Exact integer arithmetic: the tolerance is zero."""
+import numpy as np
+import pytest
+
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+RING = {"2N": 0, "3N": 3, "5N/2": 5}
+
+
+def pair(ring, logN, bits, L, alpha=1, keys=False):
+    import paper_2604_19890_gb300 as ssg
+    kw = dict(logN=logN, L=L, alpha=alpha, bits=bits, p=17, r=1, h=8, seed=23, m_odd=RING[ring])
+    g, o = ssg.Context(nmax=0, **kw), O.Oracle(**kw)
+    if keys:
+        g.keygen([])
+        o.keygen([])
+    return g, o
+
+
+@pytest.mark.parametrize("outer", [1, 2, 3, 5, 9])
+@pytest.mark.parametrize("ring,logN,bits", [("2N", 13, 55), ("2N", 14, 36), ("2N", 15, 55), ("2N", 13, 56),
+                                            ("3N", 13, 55), ("3N", 14, 55), ("5N/2", 13, 55), ("5N/2", 14, 36)])
+def test_transform_counts_and_extremes(ring, logN, bits, outer):
+    import torch
+    L = 2
+    g, o = pair(ring, logN, bits, L)
+    rng = np.random.default_rng(100 * logN + outer)
+    data = np.stack([rng.integers(0, int(g.primes[i % L]), g.N, dtype=np.uint64) for i in range(outer * L)])
+    for i in range(L):  # the first polynomials: every word q - 1; q - 1 in the upper half, in every other word
+        q = int(g.primes[i])
+        data[i] = q - 1
+        if outer > 1:
+            data[L + i] = 0
+            data[L + i, g.N // 2:] = q - 1
+        if outer > 2:
+            data[2 * L + i] = 0
+            data[2 * L + i, ::2] = q - 1
+    t = torch.from_numpy(data.view(np.int64).copy()).cuda()
+    g.ntt_forward(t, 0, L)
+    fw = t.cpu().numpy().view(np.uint64).copy()
+    for j in range(min(outer * L, 6)):
+        assert (fw[j] == o.ntt_fwd(j % L, data[j])).all(), j
+    assert (fw[-1] == o.ntt_fwd(L - 1, data[-1])).all()
+    g.ntt_inverse(t, 0, L)
+    assert (t.cpu().numpy().view(np.uint64) == data).all()
+    t = torch.from_numpy(data.view(np.int64).copy()).cuda()  # the same words as values: the inverse's own extremes
+    g.ntt_inverse(t, 0, L)
+    inv = t.cpu().numpy().view(np.uint64)
+    for j in range(min(outer * L, 6)):
+        assert (inv[j] == o.ntt_inv(j % L, data[j])).all(), j
+
+
+@pytest.mark.parametrize("count,level", [(1, 2), (3, 5), (5, 4)])
+@pytest.mark.parametrize("ring,bits", [("2N", 55), ("3N", 36), ("5N/2", 55), ("2N", 57)])
+def test_multiplication_with_ragged_digits(ring, bits, count, level):
+    """Groups of polynomials that leave out a digit's own limbs (the last digit shorter than alpha)."""
+    g, o = pair(ring, 13, bits, 5, alpha=2, keys=True)
+    rng = np.random.default_rng(count)
+    vals = rng.integers(0, g.t, (2, count, g.slots))
+    a, b = (g.encrypt(np.stack([g.encode(v) for v in vals[k]]), 10 + 20 * k) for k in (0, 1))
+    oa, ob = ([o.encrypt(o.encode(v), 10 + 20 * k + i) for i, v in enumerate(vals[k])] for k in (0, 1))
+    if level < 5:
+        a, b = g.modswitch(a, 5 - level), g.modswitch(b, 5 - level)
+        oa, ob = [o.modswitch(x, 5 - level) for x in oa], [o.modswitch(x, 5 - level) for x in ob]
+    w = g.mul_relin(a, b).words()
+    for i in (0, count - 1):
+        assert (w[i] == o.mul(oa[i], ob[i]).words()).all()
