@@ -539,6 +539,7 @@ Context::~Context() {
   cudaFree(d_pinv);
   cudaFree(d_tmod);
   cudaFree(d_tables);
+  cudaFree(d_modup);
   cudaFree(d_crt);
   cudaFree(d_sk);
   cudaFree(d_sk2);
@@ -643,6 +644,7 @@ void build_context(Context& C, const ss_params& prm) {
   }
   upload((void**)&C.d_mod, md.data(), sizeof(ModDesc) * T);
 
+  std::vector<u64> r64(4 * T, 0), fold_w1(T, 1);  // fold_w1: the forward node-1 twiddle of X^N + 1
   // twiddles: psi^brv(i) and psi^-brv(i) with Shoup companions (m = 2N; m = 3N below)
   {
     // transforms of N >= 8192 multiply by halves where the primes leave nine spare bits
@@ -652,7 +654,7 @@ void build_context(Context& C, const ss_params& prm) {
     std::vector<int> slot(halves ? N : 0);
     for (int k = 1; k < N && halves; ++k) slot[k] = ntt_tw_slot(C, k);
     std::vector<u32> tp(halves ? (size_t)T * 4 * slots : 0);
-    std::vector<u64> ninv(6 * T, 0), pinv(2 * T), r64(4 * T, 0);
+    std::vector<u64> ninv(6 * T, 0), pinv(2 * T);
     std::vector<u64> split(C.m_odd == 5 ? (size_t)T * 24 : 0);
     for (int i = 0; i < T; ++i) {
       u64 q = C.primes[i], ps = C.psi[i], pi = nt::inv(ps, q);
@@ -745,6 +747,7 @@ void build_context(Context& C, const ss_params& prm) {
           put(k, fw[rk], bw[rk]);
         }
         // 2^64 times the forward node-1 twiddle psi^bitrev(1) = psi^(N/2)
+        fold_w1[i] = fw[N / 2];
         r64[4 * i + 1] = nt::mul(r64[4 * i], fw[N / 2], q);
         // 2^64 N^-1 and 2^64 N^-1 psi^(-N/2): the inverse's last-stage factors of the lower and upper half
         r64[4 * i + 2] = nt::mul(r64[4 * i], ni, q);
@@ -878,6 +881,34 @@ void build_context(Context& C, const ss_params& prm) {
     }
   C.tables_words = tab.size();
   upload((void**)&C.d_tables, tab.data(), tab.size() * 8);
+
+  // ModUp rows (k_modup): the same constants in the form its arithmetic takes
+  if (C.d_tp && C.alpha <= 4) {
+    const int al = C.alpha, split = al < 4 ? 30 : 29;
+    const size_t words = modup_row_words(T, al);
+    std::vector<u64> mu((size_t)C.dnum * al * 2 * words, 0);
+    for (auto& kv : C.off_modup) {
+      const int j = kv.first.first, cnt = kv.first.second - j * al;
+      const u64* c1 = &tab[kv.second];
+      const u64* c2 = c1 + 2 * cnt;
+      for (int u = 0; u < 2; ++u) {
+        u64* row = &mu[((size_t)(j * al + cnt - 1) * 2 + u) * words];
+        for (int s = 0; s < cnt; ++s) {
+          const u64 qs = C.primes[j * al + s];
+          // X^N + 1: 2^64 N^-1, 2^64 N^-1 psi^(-N/2) (d_r64), the inverse's last stage; other rings 2^64
+          row[s] = nt::mul(c1[2 * s], r64[4 * (j * al + s) + (C.m_odd == 1 ? 2 + u : 0)], qs);
+          for (int g = 0; g < T; ++g) {
+            const u64 q = C.primes[g];
+            const u64 w = nt::mul(c2[(size_t)s * T + g], u && C.m_odd == 1 ? fold_w1[g] : 1, q);
+            u64* o = row + al + ((size_t)g * al + s) * 2;
+            o[0] = nt::mul(w, (1ULL << 32) % q, q);
+            o[1] = nt::mul(w, (1ULL << (32 + split)) % q, q);
+          }
+        }
+      }
+    }
+    upload((void**)&C.d_modup, mu.data(), mu.size() * 8);
+  }
 
   // decryption CRT (Garner): inverse prefix products, half-Q digits per level,
   // prefix products mod p^e.

@@ -381,6 +381,110 @@ __global__ void __launch_bounds__(256) k_bconv_many_impl(const u64* __restrict__
   }
 }
 
+// ---------------------------------------------------------------- ModUp of all digits
+// Digit j of a key switch at level l (primes [lo, hi), lo = j NS, hi = min(lo + NS,
+// l)) converted to the other data primes and the special primes, for every digit
+// in one launch. Output word: sum_s y_s c_s mod q_g, y_s = [x_s c1_s]_{q_s} exact.
+// By halves of y_s (SPLIT low bits l_s, the rest h_s): sum_s l_s c_s0 + h_s c_s1 with
+// c_s0 = c_s 2^32, c_s1 = c_s 2^(32+SPLIT) mod q_g, below (NS / 4 + ..) 2^32 q_g, and one
+// Montgomery step by 2^32; the result is below 3 q_g, as the forward transform that
+// reads it takes. SPLIT leaves the low products' sum below 2^64, so a target costs
+// 4 NS + 2 accumulating 64-bit products and one 32-bit one (58 cycles of the multiply
+// pipe a warp for NS = 3) where 128-bit sums and a Montgomery step by 2^64 took 72 and
+// 128-bit carries. The constants come from a table made with the context
+// (ModupTab), the upper half's already times the transform's node-1 twiddle.
+// One launch per digit left most SMs idle for few ciphertexts or small rings (two
+// ciphertexts at N = 2^16: 256 blocks of the 1216 that fit); when even all digits
+// do not fill the GPU, the targets of a digit are dealt to `parts` blocks.
+__device__ __forceinline__ void mac_pair(u32& a0, u32& a1, u32 x, u32 y) {
+  asm("mad.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.u32 %1, %2, %3, %1;" : "+r"(a0), "+r"(a1) : "r"(x), "r"(y));
+}
+struct ModupArgs {
+  const u64* src;  // coefficient form, [B][level][N]
+  u64* dst;        // [B][dn][level + alpha][N]
+  const u64* tab;
+  int level, L, T, N, dn, parts;
+  const ModDesc* mods;
+};
+
+template <int NS>
+__global__ void __launch_bounds__(256) k_modup_impl(const ModupArgs A) {
+  constexpr int V = 2, SPLIT = NS < 4 ? 30 : 29;
+  extern __shared__ u64 sh[];
+  const int nx = A.level + NS;
+  const int j = blockIdx.y / A.parts, part = blockIdx.y % A.parts;
+  const int lo = j * NS, hi = min(lo + NS, A.level), cnt = hi - lo;
+  const int half = 2 * V * blockIdx.x * blockDim.x >= A.N ? 1 : 0;  // block-uniform
+  // targets [0, lo) and [hi, nx) of this part, contiguous in their own numbering
+  const int nt = nx - cnt;
+  const int t0 = (int)((long)nt * part / A.parts), t1 = (int)((long)nt * (part + 1) / A.parts);
+  const u64* row = A.tab + (size_t)((lo + cnt - 1) * 2 + half) * modup_row_words(A.T, NS);
+  constexpr int W = 2 * NS + 2;  // NS pairs (c_s0, c_s1), then q and -q^-1 mod 2^64
+  for (int i = threadIdx.x; i < (t1 - t0) * W; i += blockDim.x) {
+    const int t = i / W, w = i - t * W;
+    const int m = t0 + t < lo ? t0 + t : t0 + t + cnt;
+    const int g = m < A.level ? m : A.L + (m - A.level);
+    sh[i] = w < 2 * NS ? row[NS + (size_t)g * 2 * NS + w] : w == 2 * NS ? MOD(A.mods, g).q : MOD(A.mods, g).qinv;
+  }
+  const long n = V * ((long)blockIdx.x * blockDim.x + threadIdx.x);
+  const int b = blockIdx.z;
+  u32 yl[NS][V], yh[NS][V];
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    u64 v[V] = {0, 0};
+    if (s < cnt && n < A.N) ldv<V>(A.src + ((long)b * A.level + lo + s) * A.N + n, v);
+    const Modulus& ms = MOD(A.mods, s < cnt ? lo + s : lo);
+    const u64 cm = s < cnt ? row[s] : 0;
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+      const u64 y = redc128(mulhi64(v[i], cm), v[i] * cm, ms.q, ms.qinv);
+      yl[s][i] = (u32)y & ((1u << SPLIT) - 1);
+      yh[s][i] = (u32)(y >> SPLIT);
+    }
+  }
+  __syncthreads();
+  if (n >= A.N) return;
+  u64* out = A.dst + ((long)b * A.dn + j) * nx * A.N + n;
+  for (int t = t0; t < t1; ++t) {
+    const u64* e = sh + (t - t0) * W;
+    u32 a0[V], a1[V], h0[V], h1[V];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const u64 c0 = e[2 * s], c1 = e[2 * s + 1];
+#pragma unroll
+      for (int i = 0; i < V; ++i) {
+        if (s == 0) a0[i] = a1[i] = h0[i] = h1[i] = 0;
+        mac_pair(a0[i], a1[i], yl[s][i], (u32)c0);
+        mac_pair(a0[i], a1[i], yh[s][i], (u32)c1);
+        mac_pair(h0[i], h1[i], yl[s][i], (u32)(c0 >> 32));
+        mac_pair(h0[i], h1[i], yh[s][i], (u32)(c1 >> 32));
+      }
+    }
+    const u64 q = e[2 * NS];
+    const u32 qi = (u32)e[2 * NS + 1];
+    u64 r[V];
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+      const u32 m = a0[i] * qi;
+      u32 r0, r1;
+      asm("{\n\t"
+          ".reg .u32 t0, t1, c, g0, g1;\n\t"
+          "mad.lo.cc.u32 t0, %2, %3, %5;\n\t"
+          "madc.hi.cc.u32 t1, %2, %3, %6;\n\t"
+          "addc.u32 c, 0, 0;\n\t"
+          "mad.lo.cc.u32 g0, %2, %4, %7;\n\t"
+          "madc.hi.u32 g1, %2, %4, %8;\n\t"
+          "add.cc.u32 %0, g0, t1;\n\t"
+          "addc.u32 %1, g1, c;\n\t"
+          "}"
+          : "=r"(r0), "=r"(r1)
+          : "r"(m), "r"((u32)q), "r"((u32)(q >> 32)), "r"(a0[i]), "r"(a1[i]), "r"(h0[i]), "r"(h1[i]));
+      r[i] = ((u64)r1 << 32) | r0;
+    }
+    stv<V>(out + (long)(t < lo ? t : t + cnt) * A.N, r);
+  }
+}
+
 // out[m] = (a[m] - d[m]) * scale[m] (+ add[m]); limb m is data prime m.
 __global__ void k_sub_scale_impl(const u64* a, long a_os, const u64* dl, long d_os, const u64* scale, const u64* add,
                                  long add_os, u64* out, long out_os, int nl, int N, const ModDesc* mods) {
@@ -1256,6 +1360,27 @@ void k_bconv(Context& C, const u64* src, long src_os, int ns, int sp0, const u64
   }
 #undef SS_BCONV
   kt_end(C, kr_, KC_BCONV, (double)(ns + nd - (skip_hi - skip_lo)) * n_outer * C.N * 8.0, st);
+  LAUNCHED();
+}
+
+void k_modup(Context& C, const u64* src, u64* dst, int level, int B, cudaStream_t st) {
+  const int a = C.alpha, dn = (level + a - 1) / a, nx = level + a;
+  ModupArgs A{src, dst, C.d_modup, level, C.L, C.ntot, C.N, dn, 1, C.d_mod};
+  const int bx = (C.N + 2 * TPB - 1) / (2 * TPB);
+  // four blocks of 256 threads per SM, a part of four targets at least
+  const long blocks = (long)bx * dn * B;
+  A.parts = (int)std::max(1L, std::min((4L * 152 + blocks - 1) / blocks, (long)nx / 4));
+  const dim3 g(bx, dn * A.parts, B);
+  const size_t smem = (size_t)((nx + A.parts - 1) / A.parts + 1) * (2 * a + 2) * 8;
+  if (B > 65535 || dn * A.parts > 65535) throw Error(SS_ERR_SHAPE, "too many digits or ciphertexts in one conversion");
+  int kr = kt_begin(C, st);
+  switch (a) {
+    case 1: k_modup_impl<1><<<g, TPB, smem, st>>>(A); break;
+    case 2: k_modup_impl<2><<<g, TPB, smem, st>>>(A); break;
+    case 3: k_modup_impl<3><<<g, TPB, smem, st>>>(A); break;
+    default: k_modup_impl<4><<<g, TPB, smem, st>>>(A); break;
+  }
+  kt_end(C, kr, KC_BCONV, (double)(level + dn * nx - level) * B * C.N * 8.0, st);
   LAUNCHED();
 }
 

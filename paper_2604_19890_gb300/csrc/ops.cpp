@@ -88,6 +88,23 @@ static PolySet scaled_later(PolySet s, bool post) {
   return s;
 }
 
+// ModUp of every digit: one launch where the context has its table (N >= 8192,
+// primes below 2^55, alpha <= 4), else one base conversion per digit.
+static void modup(Context& C, const u64* dc, u64* ext, int l, int B, bool pre, bool post, cudaStream_t st) {
+  if (C.d_modup) {
+    k_modup(C, dc, ext, l, B, st);
+    return;
+  }
+  const int N = C.N, a = C.alpha, dn = (l + a - 1) / a, nx = l + a;
+  for (int j = 0; j < dn; ++j) {
+    const int lo = j * a, hi = std::min(lo + a, l);
+    const u64* c1 = C.d_tables + C.off_modup.at({j, hi});
+    const u64* c2 = c1 + 2 * (hi - lo);
+    k_bconv(C, dc + (size_t)lo * N, (long)l * N, hi - lo, lo, c1, c2, ext + (size_t)j * nx * N, (long)dn * nx * N, nx, l,
+            lo, hi, nullptr, B, st, -1, pre, post);
+  }
+}
+
 // out.comp0 = addend.comp0 + KS(in.comp)[0]; out.comp1 = (addend ? addend.comp1 : 0) + KS[1]
 // addend_comp1 selects whether the addend's component 1 is added too.
 static void keyswitch_impl(Context& C, const Buf& in, int comp, const KeyDev& K, const Buf* addend, bool add_c1,
@@ -105,14 +122,7 @@ static void keyswitch_impl(Context& C, const Buf& in, int comp, const KeyDev& K,
   const long ext_os = (long)dn * nx * N;
   u64* ext = static_cast<u64*>(pool_alloc((size_t)B * ext_os * 8, st));
   const bool pre = bconv_folds_w1(C);
-  for (int j = 0; j < dn; ++j) {
-    int lo = j * a, hi = std::min(lo + a, l);
-    size_t off = C.off_modup.at({j, hi});
-    const u64* c1 = C.d_tables + off;
-    const u64* c2 = c1 + 2 * (hi - lo);
-    k_bconv(C, dc + (size_t)lo * N, (long)l * N, hi - lo, lo, c1, c2, ext + (size_t)j * nx * N, ext_os, nx, l, lo,
-            hi, nullptr, B, st, -1, pre, post);
-  }
+  modup(C, dc, ext, l, B, pre, post, st);
   PolySet ps{ext, (long)nx * N, B * dn, nx, 0, l};
   ps.skip_w = a;
   ps.skip_mod = dn;
@@ -179,13 +189,7 @@ void op_relin_drop(Context& C, const Buf& in, Buf& out, cudaStream_t st) {
   const long ext_os = (long)dn * nx * N;
   u64* ext = static_cast<u64*>(pool_alloc((size_t)B * ext_os * 8, st));
   const bool pre = bconv_folds_w1(C);
-  for (int j = 0; j < dn; ++j) {
-    int lo = j * a, hi = std::min(lo + a, l);
-    const u64* c1 = C.d_tables + C.off_modup.at({j, hi});
-    const u64* c2 = c1 + 2 * (hi - lo);
-    k_bconv(C, dc + (size_t)lo * N, (long)l * N, hi - lo, lo, c1, c2, ext + (size_t)j * nx * N, ext_os, nx, l, lo,
-            hi, nullptr, B, st, -1, pre, post);
-  }
+  modup(C, dc, ext, l, B, pre, post, st);
   PolySet ps{ext, (long)nx * N, B * dn, nx, 0, l};
   ps.skip_w = a;
   ps.skip_mod = dn;

@@ -47,6 +47,9 @@ std::vector<i64> g_coeffs_reduced(int p, int e);  // equivalent, least sum of |c
 std::vector<i64> flt_coeffs(int p);       // centred mod p
 }  // namespace nt
 
+// words of one row of Context::d_modup
+__host__ __device__ inline size_t modup_row_words(int T, int alpha) { return (size_t)alpha * (1 + 2 * (size_t)T); }
+
 // Modulus descriptor shared with device code (layout matches Modulus in modarith.cuh)
 struct ModDesc {
   u64 q, mu;
@@ -145,6 +148,11 @@ struct Context {
   u64* d_tmod = nullptr;              // [r+1][ntot][2]: p^e mod q, shoup
   u64* d_tables = nullptr;            // base-conversion constants (offsets below)
   size_t tables_words = 0;
+  // ModUp of all digits in one launch (transforms by halves, alpha <= 4; else null): for digit j of cnt primes and
+  // half u, row (j alpha + cnt - 1) 2 + u of modup_row_words words: c1_s times 2^64 and the inverse's deferred
+  // factor of that half [alpha], then per prime g the pairs (c_s 2^32, c_s 2^(32+SPLIT)) [alpha], times the
+  // node-1 twiddle in the upper half of X^N + 1
+  u64* d_modup = nullptr;
   // ModUp: key (j, e) -> offset of c1[k], c1s[k], c2[k][ntot]
   std::map<std::pair<int, int>, size_t> off_modup;
   // ModDown: t_exp -> offset of c1[alpha], c1s[alpha]; c2 [alpha][ntot]; Pinv[ntot][2]
@@ -261,6 +269,9 @@ void k_tensor(Context& C, const Buf& a, const Buf& b, Buf& out, cudaStream_t st)
 void k_bconv(Context& C, const u64* src, long src_os, int ns, int sp0, const u64* c1, const u64* c2, u64* dst,
              long dst_os, int nd, int nq, int skip_lo, int skip_hi, const u64* post, int n_outer, cudaStream_t st,
              int nsq = -1, bool pre_w1 = false, bool post_scale = false);
+// every digit of [B][level][N] (coefficient form, the inverse's last stage deferred on X^N + 1) to the extended
+// basis, [B][dnum][level + alpha][N] (node-1 twiddle applied on X^N + 1); needs C.d_modup
+void k_modup(Context& C, const u64* src, u64* dst, int level, int B, cudaStream_t st);
 // acc_c[acc_limb] += P * d_c[l-1] (acc: nx limbs per component)
 void k_fixup_last(Context& C, u64* acc, long acc_os, int nx, int acc_limb, const Buf& d, int l, const u64* pmod,
                   int B, cudaStream_t st);
