@@ -71,3 +71,31 @@ def test_multiplication_with_ragged_digits(ring, bits, count, level):
     w = g.mul_relin(a, b).words()
     for i in (0, count - 1):
         assert (w[i] == o.mul(oa[i], ob[i]).words()).all()
+
+
+@pytest.mark.parametrize("nin,nout", [(1, 1), (2, 16), (7, 3), (15, 8), (16, 16)])
+@pytest.mark.parametrize("bits,logN", [(36, 9), (55, 13), (58, 8)])
+def test_small_coefficient_combinations(bits, logN, nin, nout):
+    """sum_i c_i y_i with |c_i| < 2^27: the largest sums of each sign, words q - 1, zeros, and rows one past the bound."""
+    import paper_2604_19890_gb300 as ssg
+    g = ssg.Context(logN=logN, L=3, alpha=1, bits=bits, p=17, r=1, h=8, seed=5, nmax=0)
+    rng = np.random.default_rng(nin)
+    level, top = 2, (1 << 27) - 1
+    w = np.stack([np.stack([rng.integers(0, int(g.primes[i]), (1, 2, g.N), dtype=np.uint64) for i in range(level)], 2)
+                  for _ in range(nin)])  # [nin][1][2][level][N]
+    for i in range(level):
+        w[:, 0, 0, i, ::3] = int(g.primes[i]) - 1
+        w[:, 0, 1, i, ::5] = 0
+    rows = rng.integers(-top, top + 1, (nout, nin))
+    rows[0] = top
+    rows[-1] = -top
+    if nout > 2:
+        rows[1, 0] = 0
+        rows[2, -1] = top + 1 if nin == 7 else top  # 2^27 takes the wider path for the whole call
+    outs = g.linear_combinations([g.from_words(x, 1) for x in w], rows.tolist())
+    for j in (0, nout - 1, nout // 2):
+        got = outs[j].words()[0]
+        for i in range(level):
+            q = int(g.primes[i])
+            exp = sum(int(rows[j, t]) * w[t, 0, :, i, :].astype(object) for t in range(nin)) % q
+            assert (got[:, i, :].astype(object) == exp).all(), (j, i)
