@@ -228,6 +228,7 @@ static void run_lanes(ss_batch& b, cudaStream_t st) {
   for (int k = 0; k < n; ++k)
     th.emplace_back([&, k] {
       cudaSetDevice(dev);
+      PlainLaunches plain(true);
       LaneMerger::t_lane = k;
       ntt_merger() = &M;
       ks_merger() = &M;
@@ -263,6 +264,7 @@ static void run_all(ss_batch& b, cudaStream_t st) {
   cudaEvent_t fork = b.events[b.nstreams];
   SS_CUDA(cudaEventRecord(fork, st));
   for (int k = 0; k < b.nstreams; ++k) SS_CUDA(cudaStreamWaitEvent(b.streams[k], fork, 0));
+  PlainLaunches plain(b.nstreams > 1);
   int rr = 0;
   for (auto& g : b.groups)
     for (int i0 = 0; i0 < (int)g.items.size(); i0 += b.chunk) {

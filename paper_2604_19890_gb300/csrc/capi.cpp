@@ -1,5 +1,6 @@
 // extern "C" entry points declared in include/ss.h. Every entry point catches
 // library errors and returns them as ss_status; the message is kept per thread.
+#include <algorithm>
 #include <cstring>
 #include <string>
 
@@ -331,10 +332,16 @@ ss_status ss_mul_relin(ss_ctx* ctx, const ss_ct* a, const ss_ct* b, ss_ct* out, 
     check_ct(ctx->C, a, "null a");
     check_ct(ctx->C, b, "null b");
     need(a->count == b->count, SS_ERR_SHAPE, "batch sizes differ");
-    auto r = ss::plan_then_run(ctx->C, [&] {
-      return ss::ev_mul(ctx->C, ss::view_buf(*a), ss::view_buf(*b), S(stream));
-    });
-    deliver(ctx->C, r, out, S(stream));
+    ss::BufP va = ss::view_buf(*a), vb = ss::view_buf(*b);
+    ss::Buf plan;
+    {
+      ss::PlanScope ps(ctx->C);
+      ss::ev_mul_into(ctx->C, va, vb, plan, S(stream));
+    }
+    check_out(out, a->count, 2, std::min(a->level, b->level) - 1);
+    ss::Buf o = as_out(out);
+    ss::ev_mul_into(ctx->C, va, vb, o, S(stream));
+    write_back(o, out);
   });
 }
 

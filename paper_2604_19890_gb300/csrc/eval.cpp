@@ -112,19 +112,29 @@ BufP ev_lincomb(Context& C, const std::vector<std::pair<BufP, i64>>& terms, i64 
   return acc;
 }
 
-BufP ev_mul(Context& C, const BufP& a0, const BufP& b0, cudaStream_t st) {
+// level of the product's operands
+static int mul_level(const BufP& a0, const BufP& b0) {
   same_t(a0, b0);
   if (a0->ncomp != 2 || b0->ncomp != 2) throw Error(SS_ERR_SHAPE, "multiplication needs 2-component inputs");
   int l = std::min(a0->level, b0->level);
   if (l < 2) throw Error(SS_ERR_NOISE, "the plan needs more levels than the chain has");
+  return l;
+}
+
+void ev_mul_into(Context& C, const BufP& a0, const BufP& b0, Buf& out, cudaStream_t st) {
+  const int l = mul_level(a0, b0);
   BufP a = ev_modswitch_to(C, a0, l, st), b = ev_modswitch_to(C, b0, l, st);
   if (a->count != b->count) throw Error(SS_ERR_SHAPE, "batch sizes differ");
   BufP t3 = alloc_buf(C, a->count, 3, l, a->t_exp, st);
-  BufP out = alloc_buf(C, a->count, 2, l - 1, a->t_exp, st);
   if (!is_dry(C)) {
     k_tensor(C, *a, *b, *t3, st);
-    op_relin_drop(C, *t3, *out, st);
+    op_relin_drop(C, *t3, out, st);
   }
+}
+
+BufP ev_mul(Context& C, const BufP& a0, const BufP& b0, cudaStream_t st) {
+  BufP out = alloc_buf(C, a0->count, 2, mul_level(a0, b0) - 1, a0->t_exp, st);
+  ev_mul_into(C, a0, b0, *out, st);
   return out;
 }
 

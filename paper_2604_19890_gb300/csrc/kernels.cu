@@ -10,6 +10,7 @@
 #include <cstring>
 #include <atomic>
 
+#include "launch.cuh"
 #include "modarith.cuh"
 #include "philox.h"
 #include "ss_internal.h"
@@ -113,6 +114,7 @@ dim3 grid_for(int N, int polys) {
 // ---------------------------------------------------------------- add / sub
 __global__ void k_binary_impl(int op, const u64* a, const u64* b, u64* out, int N, int ncomp, int level, int acap,
                               int bcap, int ocap, int bcast, const ModDesc* mods) {
+  enter_grid();
   int poly = blockIdx.y;  // (bt, c, i)
   int i = poly % level, c = (poly / level) % ncomp, bt = poly / (level * ncomp);
   int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -129,6 +131,7 @@ __global__ void k_binary_impl(int op, const u64* a, const u64* b, u64* out, int 
 // ---------------------------------------------------------------- scalars
 __global__ void k_scalar_impl(int op, const u64* a, i64 c, u64* out, int N, int ncomp, int level, int acap,
                               int ocap, const ModDesc* mods, const u64* pinv) {
+  enter_grid();
   __shared__ u64 sw[2];
   int poly = blockIdx.y;
   int i = poly % level, comp = (poly / level) % ncomp, bt = poly / (level * ncomp);
@@ -172,6 +175,7 @@ __global__ void k_copy_impl(const u64* a, u64* out, int N, int ncomp, int level,
 // ---------------------------------------------------------------- tensor
 __global__ void k_tensor_impl(const u64* a, const u64* b, u64* out, int N, int level, int acap, int bcap, int ocap,
                               const ModDesc* mods) {
+  enter_grid();
   int poly = blockIdx.y;  // (bt, i)
   int i = poly % level, bt = poly / level;
   int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -219,12 +223,13 @@ __global__ void k_tensor_impl(const u64* a, const u64* b, u64* out, int N, int l
 // Montgomery form (staged per block after the targets' rows) and a Montgomery
 // reduction in place of the Shoup product, which accepts any 64-bit word.
 template <int NS, int V>
-__global__ void __launch_bounds__(256) k_bconv_impl(const u64* __restrict__ src, long src_os, int ns, int sp0, int nsq,
+__global__ void __launch_bounds__(256) k_bconv_impl(const u64* src, long src_os, int ns, int sp0, int nsq,
                                                     const u64* __restrict__ c1, const u64* __restrict__ c2, int T,
                                                     u64* __restrict__ dst, long dst_os, int nd, int nq, int L,
                                                     int skip_lo, int skip_hi, const u64* __restrict__ post, int N,
                                                     const ModDesc* mods, const u64* __restrict__ r64, int pre,
                                                     int dscale) {
+  enter_grid();
   extern __shared__ u64 sh[];
   const int ns_ = NS > 0 ? NS : ns;
   const int W = 2 + ns_;
@@ -304,12 +309,13 @@ __global__ void __launch_bounds__(256) k_bconv_impl(const u64* __restrict__ src,
 // node-1 twiddle folded into the upper half, dscale: the inverse's deferred last
 // stage folded into the source constants, as in k_bconv_impl.
 template <int TC, int V>
-__global__ void __launch_bounds__(256) k_bconv_many_impl(const u64* __restrict__ src, long src_os, int ns, int sp0,
+__global__ void __launch_bounds__(256) k_bconv_many_impl(const u64* src, long src_os, int ns, int sp0,
                                                          int nsq, const u64* __restrict__ c1,
                                                          const u64* __restrict__ c2, int T, u64* __restrict__ dst,
                                                          long dst_os, int nd, int nq, int L, int skip_lo, int skip_hi,
                                                          const u64* __restrict__ post, int N, const ModDesc* mods,
                                                          const u64* __restrict__ r64, int pre, int dscale) {
+  enter_grid();
   extern __shared__ u64 sh[];
   const int W = 2 + ns;
   const int half = 2 * V * blockIdx.x * blockDim.x >= N ? 1 : 0;  // block-uniform
@@ -411,6 +417,7 @@ struct ModupArgs {
 
 template <int NS>
 __global__ void __launch_bounds__(256) k_modup_impl(const ModupArgs A) {
+  enter_grid();
   constexpr int V = 2, SPLIT = NS < 4 ? 30 : 29;
   extern __shared__ u64 sh[];
   const int nx = A.level + NS;
@@ -490,6 +497,7 @@ __global__ void __launch_bounds__(256) k_modup_impl(const ModupArgs A) {
 // out[m] = (a[m] - d[m]) * scale[m] (+ add[m]); limb m is data prime m.
 __global__ void k_sub_scale_impl(const u64* a, long a_os, const u64* dl, long d_os, const u64* scale, const u64* add,
                                  long add_os, u64* out, long out_os, int nl, int N, const ModDesc* mods) {
+  enter_grid();
   int poly = blockIdx.y;
   int m = poly % nl, o = poly / nl;
   int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -662,7 +670,8 @@ struct KsJob {
 // are stored times 2^64 mod q and a sum is below dn q^2 < q 2^64).
 //  TYPE 0: acc[comp][m - m0] = sum_j ext_j[m] * key_j[comp][g(m)] for the limbs
 //          m = m0 + by of the extended basis (data primes, then special
-//          primes); acc holds acc_nl limbs per component.
+//          primes); acc holds acc_nl limbs per component. With x given, limb level - 1
+//          also takes P x_c (the last data limb of the relinearise-and-drop).
 //  TYPE 1, 2: the data limb m = by with the ModDown epilogue fused, so these
 //          limbs of the sum never reach memory. With acc_c[m] the reduced sum
 //          and delta_c[m] the converted correction ([ciphertext][2][nl][N],
@@ -705,6 +714,17 @@ __device__ __forceinline__ void ks_block(const KsJob& J, int bx, int by) {
         for (int v = 0; v < V; ++v) {
           r0[v] = redc128(s0[b][v].hi, s0[b][v].lo, md.q, md.qinv);
           r1[v] = redc128(s1[b][v].hi, s1[b][v].lo, md.q, md.qinv);
+        }
+        if (J.x != nullptr && m == J.level - 1) {  // relinearise and drop: the extended ciphertext's P x_c joins here
+          const u64 pw = __ldg(J.pm + 2 * m), pwp = __ldg(J.pm + 2 * m + 1);
+          u64 x0[V], x1[V];
+          ldv<V>(J.x + (long)(o0 + b) * J.x_os + (long)m * N + n, x0);
+          ldv<V>(J.x + (long)(o0 + b) * J.x_os + ((long)J.x_cap + m) * N + n, x1);
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            r0[v] = add_mod(r0[v], shoup(x0[v], pw, pwp, md.q), md.q);
+            r1[v] = add_mod(r1[v], shoup(x1[v], pw, pwp, md.q), md.q);
+          }
         }
         stv<V>(out + b * J.acc_os, r0);
         stv<V>(out + b * J.acc_os + (long)J.acc_nl * N, r1);
@@ -754,6 +774,7 @@ __global__ void __launch_bounds__(256, SS_KSIP_MINB) k_ks_ip_impl(const __grid_c
 // dynamic shared memory: SS_KSIP_STAGES slots x (2 + OB) rows x 256 threads x 16 bytes
 template <int OB, int TYPE>
 __global__ void __launch_bounds__(256, SS_KSIP_ASYNC_MINB) k_ks_ip_async(const __grid_constant__ KsJob J) {
+  enter_grid();
   ks_block<OB, TYPE, SS_KSIP_STAGES>(J, blockIdx.x, blockIdx.y);
 }
 
@@ -793,6 +814,7 @@ __global__ void __launch_bounds__(256, SS_KSIP_MINB) k_ks_ip_multi(const __grid_
 template <int RING>
 __global__ void k_automorph_impl(const u64* a, u64* out, int g, int N, int logN, int nrows, int acap, int ocap,
                                  int level) {
+  enter_grid();
   int poly = blockIdx.y;  // (bt*ncomp + c, i)
   int i = poly % level, row = poly / level;
   int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -966,6 +988,7 @@ struct LinArgs {
 // words are loaded before any arithmetic so the loads overlap.
 __global__ void __launch_bounds__(256) k_lincomb_impl(LinArgs A, int nterms, i64 cst, int small, int tiny, u64* out,
                                                       int ocap, int N, int ncomp, int level, const ModDesc* mods) {
+  enter_grid();
   const int poly = blockIdx.y;  // (bt, comp, i)
   const int i = poly % level, comp = (poly / level) % ncomp, bt = poly / (level * ncomp);
   const int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);  // two consecutive words per thread
@@ -1085,6 +1108,7 @@ struct LinMultiArgs {
 
 // Two consecutive words per thread.
 __global__ void __launch_bounds__(256) k_lincomb_multi_impl(LinMultiArgs A, int nin, int nout, int small, int N, int ncomp, int level, const ModDesc* mods) {
+  enter_grid();
   const int poly = blockIdx.y;  // (bt, comp, i)
   const int i = poly % level, comp = (poly / level) % ncomp, bt = poly / (level * ncomp);
   const int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -1161,6 +1185,7 @@ struct LinTinyArgs {
 template <int NT>
 __global__ void __launch_bounds__(256) k_lincomb_tiny_impl(const __grid_constant__ LinTinyArgs A, int nout, int N,
                                                            int ncomp, int level, const ModDesc* mods) {
+  enter_grid();
   const int poly = blockIdx.y;  // (bt, comp, i)
   const int i = poly % level, comp = (poly / level) % ncomp, bt = poly / (level * ncomp);
   const int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -1203,22 +1228,6 @@ __global__ void __launch_bounds__(256) k_lincomb_tiny_impl(const __grid_constant
   }
 }
 
-// acc_c[l-1] += P * d_c[l-1] (mod q_{l-1}) for c = 0, 1: the last data limb of
-// the extended ciphertext P*d + acc before it joins the dropped primes. That
-// limb is limb acc_limb of acc's nx limbs per component.
-__global__ void k_fixup_last_impl(u64* acc, long acc_os, int nx, int acc_limb, const u64* d, long d_os, int dcap,
-                                  int l, const u64* pmod, int N, const ModDesc* mods) {
-  int o = blockIdx.y;  // (bt, c)
-  int bt = o >> 1, c = o & 1;
-  int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  const int i = l - 1;
-  u64 q = MOD(mods, i).q;
-  u64* a = acc + (long)bt * acc_os + ((long)c * nx + acc_limb) * N + n;
-  u64 x = d[(long)bt * d_os + ((long)c * dcap + i) * N + n];
-  *a = add_mod(*a, shoup(x, pmod[2 * i], pmod[2 * i + 1], q), q);
-}
-
 // out[g] = a[g]^2 for every prime g (evaluation form)
 __global__ void k_square_impl(const u64* a, u64* out, int N, const ModDesc* mods) {
   int g = blockIdx.y;
@@ -1231,6 +1240,7 @@ __global__ void k_square_impl(const u64* a, u64* out, int N, const ModDesc* mods
 // out[c][i] = sum_b a[b][c][i]
 __global__ void k_batch_sum_impl(const u64* a, u64* out, int count, int ncomp, int level, int acap, int ocap, int N,
                                  const ModDesc* mods) {
+  enter_grid();
   int poly = blockIdx.y;  // (c, i)
   int i = poly % level, c = poly / level;
   int n = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1244,15 +1254,6 @@ __global__ void k_batch_sum_impl(const u64* a, u64* out, int count, int ncomp, i
 }  // namespace
 
 // ======================================================================= launchers
-void k_fixup_last(Context& C, u64* acc, long acc_os, int nx, int acc_limb, const Buf& d, int l, const u64* pmod,
-                  int B, cudaStream_t st) {
-  TIMED(KC_ELEM, 3.0 * 2 * B * C.N * 8.0,
-        k_fixup_last_impl<<<grid_for(C.N, 2 * B), TPB, 0, st>>>(acc, acc_os, nx, acc_limb, d.data,
-                                                                 (long)d.ncomp * d.cap * C.N, d.cap, l, pmod, C.N,
-                                                                 C.d_mod));
-  LAUNCHED();
-}
-
 void k_square(Context& C, const u64* a, u64* out, int nprimes, cudaStream_t st) {
   k_square_impl<<<grid_for(C.N, nprimes), TPB, 0, st>>>(a, out, C.N, C.d_mod);
   ++C.launches;
@@ -1287,7 +1288,7 @@ void k_lincomb(Context& C, const std::vector<const Buf*>& ys, const std::vector<
   }
   int polys = out.count * out.ncomp * out.level;
   TIMED(KC_ELEM, (nt + 1.0) * polys * C.N * 8.0,
-        k_lincomb_impl<<<grid_for(C.N / 2, polys), TPB, 0, st>>>(A, nt, cst, small ? npos + 1 : 0, tiny ? 1 : 0, out.data,
+        launch_early(k_lincomb_impl, grid_for(C.N / 2, polys), TPB, 0, st, A, nt, cst, small ? npos + 1 : 0, tiny ? 1 : 0, out.data,
                                                                   out.cap, C.N,
                                                               out.ncomp, out.level, C.d_mod));
   LAUNCHED();
@@ -1323,7 +1324,7 @@ void k_lincomb_multi(Context& C, const std::vector<const Buf*>& ys, const std::v
   const double bytes = (double)(nin + nout) * polys * C.N * 8.0;
   if (!tiny) {
     TIMED(KC_ELEM, bytes,
-          k_lincomb_multi_impl<<<grid_for(C.N / 2, polys), TPB, 0, st>>>(A, nin, nout, small ? 1 : 0, C.N, o0.ncomp,
+          launch_early(k_lincomb_multi_impl, grid_for(C.N / 2, polys), TPB, 0, st, A, nin, nout, small ? 1 : 0, C.N, o0.ncomp,
                                                                         o0.level, C.d_mod));
     LAUNCHED();
     return;
@@ -1338,7 +1339,7 @@ void k_lincomb_multi(Context& C, const std::vector<const Buf*>& ys, const std::v
   const dim3 g = grid_for(C.N / 2, polys);
   int kr = kt_begin(C, st);
 #define SS_LT(NT) \
-  case NT: k_lincomb_tiny_impl<NT><<<g, TPB, 0, st>>>(Y, nout, C.N, o0.ncomp, o0.level, C.d_mod); break;
+  case NT: launch_early(k_lincomb_tiny_impl<NT>, g, TPB, 0, st, Y, nout, C.N, o0.ncomp, o0.level, C.d_mod); break;
   switch (nin) {
     SS_LT(1) SS_LT(2) SS_LT(3) SS_LT(4) SS_LT(5) SS_LT(6) SS_LT(7) SS_LT(8)
     SS_LT(9) SS_LT(10) SS_LT(11) SS_LT(12) SS_LT(13) SS_LT(14) SS_LT(15) SS_LT(16)
@@ -1349,7 +1350,7 @@ void k_lincomb_multi(Context& C, const std::vector<const Buf*>& ys, const std::v
 }
 
 void k_batch_sum(Context& C, const Buf& a, Buf& out, cudaStream_t st) {
-  k_batch_sum_impl<<<grid_for(C.N, a.ncomp * a.level), TPB, 0, st>>>(a.data, out.data, a.count, a.ncomp, a.level,
+  launch_early(k_batch_sum_impl, grid_for(C.N, a.ncomp * a.level), TPB, 0, st, a.data, out.data, a.count, a.ncomp, a.level,
                                                                       a.cap, out.cap, C.N, C.d_mod);
   ++C.launches;
   SS_CUDA(cudaGetLastError());
@@ -1360,7 +1361,7 @@ void k_batch_sum(Context& C, const Buf& a, Buf& out, cudaStream_t st) {
 void k_binary(Context& C, int op, const Buf& a, const Buf& b, Buf& out, cudaStream_t st) {
   int polys = a.count * a.ncomp * a.level;
   TIMED(KC_ELEM, 3.0 * polys * (double)C.N * 8.0,
-  k_binary_impl<<<grid_for(C.N / 2, polys), TPB, 0, st>>>(op, a.data, b.data, out.data, C.N, a.ncomp, a.level, a.cap,
+  launch_early(k_binary_impl, grid_for(C.N / 2, polys), TPB, 0, st, op, a.data, b.data, out.data, C.N, a.ncomp, a.level, a.cap,
                                                        b.cap, out.cap, b.count == 1 && a.count > 1, C.d_mod));
   LAUNCHED();
 }
@@ -1368,7 +1369,7 @@ void k_binary(Context& C, int op, const Buf& a, const Buf& b, Buf& out, cudaStre
 void k_scalar(Context& C, int op, const Buf& a, i64 c, Buf& out, cudaStream_t st) {
   int polys = a.count * a.ncomp * a.level;
   TIMED(KC_ELEM, 2.0 * polys * (double)C.N * 8.0,
-  k_scalar_impl<<<grid_for(C.N / 2, polys), TPB, 0, st>>>(op, a.data, c, out.data, C.N, a.ncomp, a.level, a.cap,
+  launch_early(k_scalar_impl, grid_for(C.N / 2, polys), TPB, 0, st, op, a.data, c, out.data, C.N, a.ncomp, a.level, a.cap,
                                                        out.cap, C.d_mod, C.d_pinv));
   LAUNCHED();
 }
@@ -1383,7 +1384,7 @@ void k_copy_limbs(Context& C, const Buf& a, Buf& out, int level, cudaStream_t st
 void k_tensor(Context& C, const Buf& a, const Buf& b, Buf& out, cudaStream_t st) {
   int polys = a.count * a.level;
   TIMED(KC_TENSOR, 7.0 * polys * (double)C.N * 8.0,
-  k_tensor_impl<<<grid_for(C.N / 2, polys), TPB, 0, st>>>(a.data, b.data, out.data, C.N, a.level, a.cap, b.cap, out.cap,
+  launch_early(k_tensor_impl, grid_for(C.N / 2, polys), TPB, 0, st, a.data, b.data, out.data, C.N, a.level, a.cap, b.cap, out.cap,
                                                        C.d_mod));
   LAUNCHED();
 }
@@ -1403,7 +1404,7 @@ void k_bconv(Context& C, const u64* src, long src_os, int ns, int sp0, const u64
   if (smem > 48 * 1024) throw Error(SS_ERR_PARAM, "base conversion tables exceed 48 KiB of shared memory");
   int kr_ = kt_begin(C, st);
 #define SS_BCONV(NSV, VV)                                                                                        \
-  k_bconv_impl<NSV, VV><<<dim3((g.x + VV - 1) / VV, g.y), TPB, smem, st>>>(                                       \
+  launch_early(k_bconv_impl<NSV, VV>, dim3((g.x + VV - 1) / VV, g.y), TPB, smem, st,                                        \
       src, src_os, ns, sp0, nsq, c1, c2, C.ntot, dst, dst_os, nd, nq, C.L, skip_lo, skip_hi, post, C.N, C.d_mod,     \
       C.d_r64, pre, dscale)
   switch (ns) {
@@ -1412,7 +1413,7 @@ void k_bconv(Context& C, const u64* src, long src_os, int ns, int sp0, const u64
     case 3: SS_BCONV(3, SS_BCONV_V); break;
     case 4: SS_BCONV(4, SS_BCONV_V); break;
     default:
-      k_bconv_many_impl<4, 2><<<dim3((g.x + 1) / 2, g.y), TPB, smem, st>>>(
+      launch_early(k_bconv_many_impl<4, 2>, dim3((g.x + 1) / 2, g.y), TPB, smem, st, 
           src, src_os, ns, sp0, nsq, c1, c2, C.ntot, dst, dst_os, nd, nq, C.L, skip_lo, skip_hi, post, C.N, C.d_mod,
           C.d_r64, pre, dscale);
       break;
@@ -1434,10 +1435,10 @@ void k_modup(Context& C, const u64* src, u64* dst, int level, int B, cudaStream_
   if (B > 65535 || dn * A.parts > 65535) throw Error(SS_ERR_SHAPE, "too many digits or ciphertexts in one conversion");
   int kr = kt_begin(C, st);
   switch (a) {
-    case 1: k_modup_impl<1><<<g, TPB, smem, st>>>(A); break;
-    case 2: k_modup_impl<2><<<g, TPB, smem, st>>>(A); break;
-    case 3: k_modup_impl<3><<<g, TPB, smem, st>>>(A); break;
-    default: k_modup_impl<4><<<g, TPB, smem, st>>>(A); break;
+    case 1: launch_early(k_modup_impl<1>, g, TPB, smem, st, A); break;
+    case 2: launch_early(k_modup_impl<2>, g, TPB, smem, st, A); break;
+    case 3: launch_early(k_modup_impl<3>, g, TPB, smem, st, A); break;
+    default: launch_early(k_modup_impl<4>, g, TPB, smem, st, A); break;
   }
   kt_end(C, kr, KC_BCONV, (double)(level + dn * nx - level) * B * C.N * 8.0, st);
   LAUNCHED();
@@ -1446,7 +1447,7 @@ void k_modup(Context& C, const u64* src, u64* dst, int level, int B, cudaStream_
 void k_sub_scale(Context& C, const u64* a, long a_os, const u64* dl, long d_os, const u64* scale, const u64* add,
                  long add_os, u64* out, long out_os, int nl, int n_outer, cudaStream_t st) {
   TIMED(KC_SUBSCALE, (add ? 4.0 : 3.0) * nl * n_outer * (double)C.N * 8.0,
-  k_sub_scale_impl<<<grid_for(C.N / 2, nl * n_outer), TPB, 0, st>>>(a, a_os, dl, d_os, scale, add, add_os, out, out_os,
+  launch_early(k_sub_scale_impl, grid_for(C.N / 2, nl * n_outer), TPB, 0, st, a, a_os, dl, d_os, scale, add, add_os, out, out_os,
                                                                  nl, C.N, C.d_mod));
   LAUNCHED();
 }
@@ -1508,9 +1509,9 @@ static void ks_launch(Context& C, const KsJob& J, int nlimbs, double bytes, cuda
     }
   }
   switch (J.type) {
-    case 0: TIMED(KC_KSIP, bytes, (k_ks_ip_async<OB, 0><<<grid, TPB, ring, st>>>(J))); break;
-    case 1: TIMED(KC_KSIP, bytes, (k_ks_ip_async<OB, 1><<<grid, TPB, ring, st>>>(J))); break;
-    default: TIMED(KC_KSIP, bytes, (k_ks_ip_async<OB, 2><<<grid, TPB, ring, st>>>(J))); break;
+    case 0: TIMED(KC_KSIP, bytes, (launch_early(k_ks_ip_async<OB, 0>, grid, TPB, ring, st, J))); break;
+    case 1: TIMED(KC_KSIP, bytes, (launch_early(k_ks_ip_async<OB, 1>, grid, TPB, ring, st, J))); break;
+    default: TIMED(KC_KSIP, bytes, (launch_early(k_ks_ip_async<OB, 2>, grid, TPB, ring, st, J))); break;
   }
 #else
   switch (J.type) {
@@ -1523,7 +1524,7 @@ static void ks_launch(Context& C, const KsJob& J, int nlimbs, double bytes, cuda
 }
 
 void k_ks_ip(Context& C, const u64* d, long d_os, const u64* ext, long ext_os, const KeyDev& K, int level, u64* acc,
-             long acc_os, int n_outer, cudaStream_t st, int m0, int nlimbs) {
+             long acc_os, int n_outer, cudaStream_t st, int m0, int nlimbs, const Buf* x, const u64* pm) {
   const int dn = (level + C.alpha - 1) / C.alpha;
   if (nlimbs < 0) nlimbs = level + C.alpha - m0;
   KsJob J = ks_job(C, 0, d, d_os, ext, ext_os, K, level, n_outer, nlimbs);
@@ -1531,6 +1532,10 @@ void k_ks_ip(Context& C, const u64* d, long d_os, const u64* ext, long ext_os, c
   J.acc_os = acc_os;
   J.m0 = m0;
   J.acc_nl = nlimbs;
+  J.x = x ? x->data : nullptr;
+  J.x_os = x ? (long)x->ncomp * x->cap * C.N : 0;
+  J.x_cap = x ? x->cap : 0;
+  J.pm = pm;
   // each key limb is read once per launch; ext limbs and the sums once per ciphertext
   ks_launch(C, J, nlimbs, ((double)dn * nlimbs * (n_outer + 2.0) + 2.0 * nlimbs * n_outer) * (double)C.N * 8.0, st);
 }
@@ -1595,11 +1600,11 @@ void ks_multi(const std::vector<KsReq>& reqs, cudaStream_t st) {
 void k_automorph(Context& C, const Buf& a, int g, Buf& out, cudaStream_t st) {
   int rows = a.count * a.ncomp;
   TIMED(KC_AUTOMORPH, 2.0 * rows * a.level * (double)C.N * 8.0,
-  if (C.m_odd == 5) k_automorph_impl<5><<<grid_for(C.N, rows * a.level), TPB, 0, st>>>(
+  if (C.m_odd == 5) launch_early(k_automorph_impl<5>, grid_for(C.N, rows * a.level), TPB, 0, st, 
       a.data, out.data, g, C.N, C.logN, rows, a.cap, out.cap, a.level);
-  else if (C.m_odd == 3) k_automorph_impl<3><<<grid_for(C.N, rows * a.level), TPB, 0, st>>>(
+  else if (C.m_odd == 3) launch_early(k_automorph_impl<3>, grid_for(C.N, rows * a.level), TPB, 0, st, 
       a.data, out.data, g, C.N, C.logN, rows, a.cap, out.cap, a.level);
-  else k_automorph_impl<1><<<grid_for(C.N, rows * a.level), TPB, 0, st>>>(
+  else launch_early(k_automorph_impl<1>, grid_for(C.N, rows * a.level), TPB, 0, st, 
       a.data, out.data, g, C.N, C.logN, rows, a.cap, out.cap, a.level));
   LAUNCHED();
 }

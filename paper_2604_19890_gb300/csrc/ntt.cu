@@ -18,6 +18,7 @@
 //    and 0.573 inverse, where the Shoup form takes 0.751 and 0.870.
 //  * N >= 8192, wider primes: k_ntt16 (Shoup products: halves need nine spare bits).
 //  * N <= 4096: k_ntt, one phase in shared memory with Harvey's lazy butterflies.
+#include "launch.cuh"
 #include "modarith.cuh"
 #include "ss_internal.h"
 
@@ -846,6 +847,7 @@ constexpr size_t col_smem() {
 
 template <bool FWD, int LOGS, int LOG2N, int CL, int RING>
 __global__ void __launch_bounds__(128, FWD ? SS_COLS_F : SS_COLS_I) k_ntt16_cols(NttArgs A) {
+  enter_grid();
   ntt16_cols<FWD, LOGS, LOG2N, CL, RING>(A, blockIdx.x, blockIdx.y);
 }
 
@@ -1003,6 +1005,7 @@ __device__ __forceinline__ void ntt16_rows(const NttArgs& A, const RowPlan& R, i
 
 template <bool FWD, int LOGS, bool SRC>
 __global__ void __launch_bounds__(128, FWD ? SS_ROWS_F : SS_ROWS_I) k_ntt16_rows(NttArgs A, RowPlan R) {
+  enter_grid();
   ntt16_rows<FWD, LOGS, SRC>(A, R, blockIdx.x, blockIdx.y);
 }
 
@@ -1075,7 +1078,7 @@ __global__ void __launch_bounds__(128, 6) k_ntt16_multi(const __grid_constant__ 
 template <bool FWD, int LOGS, int LOG2N, int RING>
 void launch_cols_as(int npoly, cudaStream_t st, const NttArgs& A) {
   constexpr int CL = kColTile - LOGS;
-  k_ntt16_cols<FWD, LOGS, LOG2N, CL, RING><<<dim3(1 << (LOG2N - CL), npoly), 128, col_smem<LOGS, CL>(), st>>>(A);
+  launch_early(k_ntt16_cols<FWD, LOGS, LOG2N, CL, RING>, dim3(1 << (LOG2N - CL), npoly), 128, col_smem<LOGS, CL>(), st, A);
 }
 template <bool FWD>
 void launch_cols(int ring, int logS, int log2n, int npoly, cudaStream_t st, const NttArgs& A) {
@@ -1136,8 +1139,8 @@ void launch_rows(int logS, const PolySet& s, cudaStream_t st, const NttArgs& A) 
   }
   const dim3 g(((A.N >> logS) / ((thr >> (logS - 4)) >> R.lnp)) * R.groups, s.nl);
   const size_t smem = row_smem(logS, thr, R.lnp);
-  if (logS == 7) k_ntt16_rows<FWD, 7, SRC><<<g, thr, smem, st>>>(A, R);
-  else k_ntt16_rows<FWD, 8, SRC><<<g, thr, smem, st>>>(A, R);
+  if (logS == 7) launch_early(k_ntt16_rows<FWD, 7, SRC>, g, thr, smem, st, A, R);
+  else launch_early(k_ntt16_rows<FWD, 8, SRC>, g, thr, smem, st, A, R);
 }
 
 // log2 of the chunk length N2 of the two-phase split: 256, except that the

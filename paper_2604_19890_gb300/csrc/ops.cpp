@@ -88,6 +88,20 @@ static PolySet scaled_later(PolySet s, bool post) {
   return s;
 }
 
+// Scratch of one key switch as one pool block (one allocation and one free instead
+// of four of each): the digits, the sums of the dropped limbs, and a region that
+// holds the digit source up to the ModUp and the correction afterwards.
+struct KsScratch {
+  u64 *ext, *acc, *dc, *delta;
+  cudaStream_t st;
+  KsScratch(size_t ext_words, size_t acc_words, size_t dc_words, size_t delta_words, cudaStream_t s) : st(s) {
+    ext = static_cast<u64*>(pool_alloc((ext_words + acc_words + std::max(dc_words, delta_words)) * 8, s));
+    acc = ext + ext_words;
+    dc = delta = acc + acc_words;
+  }
+  ~KsScratch() { pool_free(ext, st); }
+};
+
 // ModUp of every digit: one launch where the context has its table (N >= 8192,
 // primes below 2^55, alpha <= 4), else one base conversion per digit.
 static void modup(Context& C, const u64* dc, u64* ext, int l, int B, bool pre, bool post, cudaStream_t st) {
@@ -114,13 +128,13 @@ static void keyswitch_impl(Context& C, const Buf& in, int comp, const KeyDev& K,
   const long in_os = (long)in.ncomp * in.cap * N;
   const u64* d = in.data + (size_t)comp * in.cap * N;
   // 1. coefficient form of the digit source (read in place, written to dc)
-  u64* dc = static_cast<u64*>(pool_alloc((size_t)B * l * N * 8, st));
+  const long ext_os = (long)dn * nx * N, sp_os = 2L * a * N;
+  KsScratch ws((size_t)B * ext_os, (size_t)B * sp_os, (size_t)B * l * N, (size_t)2 * B * l * N, st);
+  u64 *dc = ws.dc, *ext = ws.ext, *acc = ws.acc, *delta = ws.delta;
   const bool post = bconv_folds_inverse(C);
   ntt_inverse_from(C, scaled_later(PolySet{dc, (long)l * N, B, l, 0, l}, post), d, in_os, st);
   // 2. ModUp of every digit to the other data primes and the special primes
   //    (X^N + 1: the base conversion also applies the transform's first twiddle)
-  const long ext_os = (long)dn * nx * N;
-  u64* ext = static_cast<u64*>(pool_alloc((size_t)B * ext_os * 8, st));
   const bool pre = bconv_folds_w1(C);
   modup(C, dc, ext, l, B, pre, post, st);
   PolySet ps{ext, (long)nx * N, B * dn, nx, 0, l};
@@ -129,14 +143,10 @@ static void keyswitch_impl(Context& C, const Buf& in, int comp, const KeyDev& K,
   ps.skip_level = l;
   ps.pre_w1 = pre;
   ntt_forward(C, ps, st);
-  pool_free(dc, st);
   // 3. inner product with the key on the special primes (both components)
-  const long sp_os = 2L * a * N;
-  u64* acc = static_cast<u64*>(pool_alloc((size_t)B * sp_os * 8, st));
   k_ks_ip(C, d, in_os, ext, ext_os, K, l, acc, sp_os, B, st, l, a);
   // 4. ModDown: delta = t * conv_P->Q(t^-1 acc mod P) on the data primes
   ntt_inverse(C, scaled_later(PolySet{acc, (long)a * N, 2 * B, a, C.L, 0}, post), st);
-  u64* delta = static_cast<u64*>(pool_alloc((size_t)2 * B * l * N * 8, st));
   const u64* c1 = C.d_tables + C.off_md_c1[in.t_exp];
   const u64* c2 = C.d_tables + C.off_md_c2;
   const u64* tpost = C.d_tmod + (size_t)in.t_exp * C.ntot * 2;
@@ -144,12 +154,9 @@ static void keyswitch_impl(Context& C, const Buf& in, int comp, const KeyDev& K,
   PolySet pd{delta, (long)l * N, 2 * B, l, 0, l};
   pd.pre_w1 = pre;
   ntt_forward(C, pd, st);
-  pool_free(acc, st);
   // 5. inner product on the data primes fused with out = (acc - delta) P^-1 (+ addend)
   const u64* pinv = C.d_tables + C.off_md_pinv;
   k_ks_ip_fused(C, d, in_os, ext, ext_os, K, l, l, false, addend, add_c1, delta, l, nullptr, pinv, out, B, st);
-  pool_free(ext, st);
-  pool_free(delta, st);
 }
 
 void op_keyswitch(Context& C, const Buf& in, int comp, const KeyDev& K, const Buf* addend, Buf& out,
@@ -183,11 +190,12 @@ void op_relin_drop(Context& C, const Buf& in, Buf& out, cudaStream_t st) {
   const long in_os = (long)in.ncomp * in.cap * N;
   const u64* d = in.data + (size_t)2 * in.cap * N;
   // 1-3: ModUp and inner product, as in keyswitch_impl
-  u64* dc = static_cast<u64*>(pool_alloc((size_t)B * l * N * 8, st));
+  const int ns = a + 1;  // limbs the ModDown drops
+  const long ext_os = (long)dn * nx * N, sp_os = 2L * ns * N;
+  KsScratch ws((size_t)B * ext_os, (size_t)B * sp_os, (size_t)B * l * N, (size_t)2 * B * nl * N, st);
+  u64 *dc = ws.dc, *ext = ws.ext, *acc = ws.acc, *delta = ws.delta;
   const bool post = bconv_folds_inverse(C);
   ntt_inverse_from(C, scaled_later(PolySet{dc, (long)l * N, B, l, 0, l}, post), d, in_os, st);
-  const long ext_os = (long)dn * nx * N;
-  u64* ext = static_cast<u64*>(pool_alloc((size_t)B * ext_os * 8, st));
   const bool pre = bconv_folds_w1(C);
   modup(C, dc, ext, l, B, pre, post, st);
   PolySet ps{ext, (long)nx * N, B * dn, nx, 0, l};
@@ -196,17 +204,12 @@ void op_relin_drop(Context& C, const Buf& in, Buf& out, cudaStream_t st) {
   ps.skip_level = l;
   ps.pre_w1 = pre;
   ntt_forward(C, ps, st);
-  pool_free(dc, st);
   // 3. inner product on q_{l-1} and the special primes (the limbs the ModDown drops)
-  const int ns = a + 1;
-  const long sp_os = 2L * ns * N;
-  u64* acc = static_cast<u64*>(pool_alloc((size_t)B * sp_os * 8, st));
-  k_ks_ip(C, d, in_os, ext, ext_os, C.rlk, l, acc, sp_os, B, st, l - 1, ns);
-  // 4. ModDown by q_{l-1} P: delta = t conv([t^-1 (P d + acc)]_D) on the first l-1 primes
+  //    with P d added on q_{l-1}
   const u64* pmod = C.d_tables + C.off_pmod;
-  k_fixup_last(C, acc, sp_os, ns, 0, in, l, pmod, B, st);
+  k_ks_ip(C, d, in_os, ext, ext_os, C.rlk, l, acc, sp_os, B, st, l - 1, ns, &in, pmod);
+  // 4. ModDown by q_{l-1} P: delta = t conv([t^-1 (P d + acc)]_D) on the first l-1 primes
   ntt_inverse(C, scaled_later(PolySet{acc, (long)ns * N, 2 * B, ns, l - 1, 1}, post), st);
-  u64* delta = static_cast<u64*>(pool_alloc((size_t)2 * B * nl * N * 8, st));
   const u64* c2 = C.d_tables + C.off_rd[l];
   const u64* inv = c2 + (size_t)(a + 1) * C.ntot;
   const u64* c1 = C.d_tables + C.off_rd_c1.at({l, in.t_exp});
@@ -215,12 +218,9 @@ void op_relin_drop(Context& C, const Buf& in, Buf& out, cudaStream_t st) {
   PolySet pd{delta, (long)nl * N, 2 * B, nl, 0, nl};
   pd.pre_w1 = pre;
   ntt_forward(C, pd, st);
-  pool_free(acc, st);
   // 5. inner product on the kept primes fused with the combine
   //    out_c = ((P d_c + acc_c) - delta_c) (q_{l-1} P)^-1
   k_ks_ip_fused(C, d, in_os, ext, ext_os, C.rlk, l, nl, true, &in, true, delta, nl, pmod, inv, out, B, st);
-  pool_free(ext, st);
-  pool_free(delta, st);
 }
 
 void op_modswitch(Context& C, const Buf& a, int k, Buf& out, cudaStream_t st) {
@@ -230,12 +230,11 @@ void op_modswitch(Context& C, const Buf& a, int k, Buf& out, cudaStream_t st) {
   out.ncomp = nc;
   out.level = nl;
   out.t_exp = a.t_exp;
-  u64* x = static_cast<u64*>(pool_alloc((size_t)B * nc * k * N * 8, st));
-  SS_CUDA(cudaMemcpy2DAsync(x, (size_t)k * N * 8, a.data + (size_t)nl * N, (size_t)a.cap * N * 8, (size_t)k * N * 8,
-                            (size_t)B * nc, cudaMemcpyDeviceToDevice, st));
+  u64* x = static_cast<u64*>(pool_alloc((size_t)B * nc * (k + nl) * N * 8, st));
+  u64* delta = x + (size_t)B * nc * k * N;
   const bool pre = bconv_folds_w1(C), post = bconv_folds_inverse(C);
-  ntt_inverse(C, scaled_later(PolySet{x, (long)k * N, B * nc, k, nl, k}, post), st);
-  u64* delta = static_cast<u64*>(pool_alloc((size_t)B * nc * nl * N * 8, st));
+  ntt_inverse_from(C, scaled_later(PolySet{x, (long)k * N, B * nc, k, nl, k}, post), a.data + (size_t)nl * N,
+                   (long)a.cap * N, st);
   size_t off = C.off_ms.at({l, k});
   const u64* c2 = C.d_tables + off;
   const u64* qinv = c2 + (size_t)k * C.ntot;
@@ -248,7 +247,6 @@ void op_modswitch(Context& C, const Buf& a, int k, Buf& out, cudaStream_t st) {
   k_sub_scale(C, a.data, (long)a.cap * N, delta, (long)nl * N, qinv, nullptr, 0, out.data, (long)out.cap * N, nl,
               B * nc, st);
   pool_free(x, st);
-  pool_free(delta, st);
 }
 
 void op_rotate(Context& C, const Buf& a, int g, Buf& out, cudaStream_t st) {

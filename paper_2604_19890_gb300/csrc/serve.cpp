@@ -56,6 +56,7 @@ struct Server {
 
   void worker(int w) {
     cudaStream_t st = streams[w];
+    PlainLaunches plain(streams.size() > 1);
     for (;;) {
       std::vector<std::shared_ptr<Request>> group;
       size_t bytes = 0;

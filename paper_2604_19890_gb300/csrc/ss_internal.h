@@ -199,6 +199,17 @@ void* pool_alloc(size_t bytes, cudaStream_t s);
 void pool_free(void* p, cudaStream_t s);
 
 // ------------------------------------------------------------------ launchers
+// Whether the calling thread launches without overlapping a kernel's start with
+// its predecessor's end (launch.cuh): while it feeds one of several busy streams.
+inline bool& plain_launches() {
+  static thread_local bool plain = false;
+  return plain;
+}
+struct PlainLaunches {
+  bool prev;
+  explicit PlainLaunches(bool on) : prev(plain_launches()) { plain_launches() = prev || on; }
+  ~PlainLaunches() { plain_launches() = prev; }
+};
 // Polys (o, i) at base + o*outer_stride + i*N, i < nl; global prime of limb i:
 // i < nq ? q0 + i : L + (i - nq). Limbs inside [skip_lo, skip_hi) of digit
 // (o % skip_mod) * skip_w .. are skipped when skip_w > 0 (ModUp outputs).
@@ -272,16 +283,15 @@ void k_bconv(Context& C, const u64* src, long src_os, int ns, int sp0, const u64
 // every digit of [B][level][N] (coefficient form, the inverse's last stage deferred on X^N + 1) to the extended
 // basis, [B][dnum][level + alpha][N] (node-1 twiddle applied on X^N + 1); needs C.d_modup
 void k_modup(Context& C, const u64* src, u64* dst, int level, int B, cudaStream_t st);
-// acc_c[acc_limb] += P * d_c[l-1] (acc: nx limbs per component)
-void k_fixup_last(Context& C, u64* acc, long acc_os, int nx, int acc_limb, const Buf& d, int l, const u64* pmod,
-                  int B, cudaStream_t st);
 void k_sub_scale(Context& C, const u64* a, long a_os, const u64* dl, long d_os, const u64* scale, const u64* add,
                  long add_os, u64* out, long out_os, int nl, int n_outer, cudaStream_t st);
 void k_to_montgomery(Context& C, u64* data, int npoly, cudaStream_t st);
 // key-switch inner product for the limbs [m0, m0 + nlimbs) of the extended
-// basis (nlimbs < 0: to the end); acc holds nlimbs limbs per component
+// basis (nlimbs < 0: to the end); acc holds nlimbs limbs per component. x, pm (P mod
+// q per prime): limb level - 1 also takes P x_c
 void k_ks_ip(Context& C, const u64* d, long d_os, const u64* ext, long ext_os, const KeyDev& K, int level,
-             u64* acc, long acc_os, int n_outer, cudaStream_t st, int m0 = 0, int nlimbs = -1);
+             u64* acc, long acc_os, int n_outer, cudaStream_t st, int m0 = 0, int nlimbs = -1, const Buf* x = nullptr,
+             const u64* pm = nullptr);
 // inner product over the data limbs [0, nlimbs) with the ModDown epilogue
 // (drop: relinearise-and-drop combine; else subtract, scale by P^-1, add x)
 void k_ks_ip_fused(Context& C, const u64* d, long d_os, const u64* ext, long ext_os, const KeyDev& K, int level,
@@ -325,6 +335,8 @@ size_t relin_noalloc_capacity();
 // evaluator (batched, one plan for every ciphertext of a batch)
 BufP ev_modswitch_to(Context& C, const BufP& a, int level, cudaStream_t st);
 BufP ev_mul(Context& C, const BufP& a, const BufP& b, cudaStream_t st);
+// the same into `out` (its data, count and capacity set; written by the last kernel only, so it may be an input)
+void ev_mul_into(Context& C, const BufP& a, const BufP& b, Buf& out, cudaStream_t st);
 BufP ev_add(Context& C, const BufP& a, const BufP& b, cudaStream_t st);
 BufP ev_sub(Context& C, const BufP& a, const BufP& b, cudaStream_t st);
 BufP ev_scalar(Context& C, int op, const BufP& a, i64 c, cudaStream_t st);
