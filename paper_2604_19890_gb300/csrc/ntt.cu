@@ -56,6 +56,9 @@ constexpr int TILE = 4096;  // words per CTA tile (32 KiB of shared memory)
 #ifndef SS_ROWS_I
 #define SS_ROWS_I 7
 #endif
+#ifndef SS_ROWS_IP
+#define SS_ROWS_IP 4  // CTAs of 256 threads
+#endif
 #ifndef SS_NTT_MINB_R5
 #define SS_NTT_MINB_R5 3  // m = 5N/2 column phases (the factored split fits the same 80 registers)
 #endif
@@ -751,7 +754,7 @@ __device__ __forceinline__ void ntt16_cols(const NttArgs& A, int tile, int poly)
   auto narrow_slot = [rest](int j, int blk) { return (1 << (LOGS - 1 - j)) + (blk << W) + rest; };
   const ulonglong2* spl =
       RING == 5 ? reinterpret_cast<const ulonglong2*>(A.split + (size_t)pidx * kSplitWords) : nullptr;
-  if (FWD) {
+  if constexpr (FWD) {
     int j0 = 3;
     if (RING == 5) {
 #pragma unroll
@@ -789,8 +792,7 @@ __device__ __forceinline__ void ntt16_cols(const NttArgs& A, int tile, int poly)
     for (int j = LOGS - 5; j >= 0; --j) half_stage<true>(x, j, 0, twS, tpS, hm, false, narrow_slot);
 #pragma unroll
     for (int k = 0; k < 16; ++k) col[(16 * rest + (long)k) * STRIDE] = x[k];
-    return;
-  }
+  } else {
 #pragma unroll
   for (int j = 0; j < 4; ++j) half_stage<false>(x, j, j, twS, tpS, hm, false, narrow_slot);
   half_settle(x, 4, hm);
@@ -837,6 +839,7 @@ __device__ __forceinline__ void ntt16_cols(const NttArgs& A, int tile, int poly)
   }
 #pragma unroll
   for (int k = 0; k < 16; ++k) col[(rest + (long)G * k) * STRIDE] = x[k];
+  }
 }
 
 constexpr int kColTile = 11;  // log2 words of a column tile: 128 threads
@@ -867,6 +870,38 @@ __global__ void __launch_bounds__(128, FWD ? SS_COLS_F : SS_COLS_I) k_ntt16_cols
 // read a pair of their own group, and sixteen that read one word each of one
 // group, touch all banks once
 __device__ __forceinline__ int row_swz(int r) { return r ^ (((r >> 4) & 7) << 1); }
+
+// a thread's share of its row, in linear order of pairs (words 16 lr .. 16 lr + 15)
+__device__ __forceinline__ void row_put(const u64 (&x)[16], u64* mine, int lr) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    *reinterpret_cast<ulonglong2*>(mine + row_swz(16 * lr + 2 * i)) = make_ulonglong2(x[2 * i], x[2 * i + 1]);
+}
+__device__ __forceinline__ void row_get(u64 (&x)[16], const u64* mine, int lr) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(mine + row_swz(16 * lr + 2 * i));
+    x[2 * i] = t.x;
+    x[2 * i + 1] = t.y;
+  }
+}
+// Both register rounds of a forward row: x holds words lr + (S/16) k on entry and
+// 16 lr + k, unreduced, on return. The whole warp calls it.
+template <int LOGS>
+__device__ __forceinline__ void row_forward(u64 (&x)[16], u64* mine, int lr, const ulonglong2* tw, const uint2* tp,
+                                            const HalfMod& hm) {
+  constexpr int TPR = (1 << LOGS) / 16;
+  auto wide_slot = [](int j, int blk) { return (1 << (3 - j)) + blk; };
+  auto narrow_slot = [lr](int j, int blk) { return (1 << (LOGS - 1 - j)) + (blk << (LOGS - 4)) + lr; };
+#pragma unroll
+  for (int j = 3; j >= 0; --j) half_stage<true>(x, j, 0, tw, tp, hm, false, wide_slot);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) mine[row_swz(lr + TPR * k)] = x[k];
+  __syncwarp();
+  row_get(x, mine, lr);
+#pragma unroll
+  for (int j = LOGS - 5; j >= 0; --j) half_stage<true>(x, j, 0, tw, tp, hm, false, narrow_slot);
+}
 
 struct RowPlan {
   int lnp, groups;  // log2 NP, groups of NP polynomials per limb (at most)
@@ -945,34 +980,14 @@ __device__ __forceinline__ void ntt16_rows(const NttArgs& A, const RowPlan& R, i
   // the narrow round holds words 16 lr .. 16 lr + 15, the wide round words lr + TPR k
   auto wide_slot = [](int j, int blk) { return (1 << (3 - j)) + blk; };
   auto narrow_slot = [lr](int j, int blk) { return (1 << (LOGS - 1 - j)) + (blk << LT) + lr; };
-  auto put_own = [&] {
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-      *reinterpret_cast<ulonglong2*>(mine + row_swz(16 * lr + 2 * i)) = make_ulonglong2(x[2 * i], x[2 * i + 1]);
-  };
-  auto get_own = [&] {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(mine + row_swz(16 * lr + 2 * i));
-      x[2 * i] = t.x;
-      x[2 * i + 1] = t.y;
-    }
-  };
   if (FWD) {
-#pragma unroll
-    for (int j = 3; j >= 0; --j) half_stage<true>(x, j, 0, tw, tp, hm, false, wide_slot);
-#pragma unroll
-    for (int k = 0; k < 16; ++k) mine[row_swz(lr + TPR * k)] = x[k];
-    __syncwarp();
-    get_own();
-#pragma unroll
-    for (int j = LOGS - 5; j >= 0; --j) half_stage<true>(x, j, 0, tw, tp, hm, false, narrow_slot);
+    row_forward<LOGS>(x, mine, lr, tw, tp, hm);
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
       const u64 r = reduce_half(x[k], hm), d = r - q;  // d wraps above r when r < q
       x[k] = r < d ? r : d;
     }
-    put_own();
+    row_put(x, mine, lr);
     __syncwarp();
 #pragma unroll
     for (int rw = 0; rw < RPW; ++rw) {
@@ -985,11 +1000,11 @@ __device__ __forceinline__ void ntt16_rows(const NttArgs& A, const RowPlan& R, i
       }
     }
   } else {
-    get_own();
+    row_get(x, mine, lr);
 #pragma unroll
     for (int j = 0; j < 4; ++j) half_stage<false>(x, j, j, tw, tp, hm, false, narrow_slot);
     half_settle(x, 4, hm);
-    put_own();
+    row_put(x, mine, lr);
     __syncwarp();
 #pragma unroll
     for (int k = 0; k < 16; ++k) x[k] = mine[row_swz(lr + TPR * k)];
@@ -1007,6 +1022,186 @@ template <bool FWD, int LOGS, bool SRC>
 __global__ void __launch_bounds__(128, FWD ? SS_ROWS_F : SS_ROWS_I) k_ntt16_rows(NttArgs A, RowPlan R) {
   enter_grid();
   ntt16_rows<FWD, LOGS, SRC>(A, R, blockIdx.x, blockIdx.y);
+}
+
+// ---------------------------------------------------------------- chunk phase with the key-switch inner product
+// The last forward phase of a key switch's digits fused with their inner product
+// with the key: a CTA holds one chunk of one limb for all digits of NB
+// ciphertexts (rows as in ntt16_rows, the digit whose primes hold the limb read
+// as it is), transforms the rows in shared memory and sums key times digit per
+// word, so the transformed digits never reach memory. For the data limbs the two
+// rows of the ModDown correction (its column phase done) are transformed beside
+// them and the epilogue follows (k_ks_ip's types; acc_c the reduced sum):
+//   type 0: acc_c[m] for the limbs the ModDown drops; with x, limb level - 1 also
+//           takes P x_c;
+//   type 1: out_c = (acc_c - delta_c) P^-1 (+ x_c; component 1 only if add_c1);
+//   type 2: out_c = ((P x_c + acc_c) - delta_c) (q_{l-1} P)^-1.
+// The separate inner product read 14 transformed limbs per limb and ciphertext
+// from memory beside transforms bound by the multiply pipe; here its products (32
+// pipe cycles a digit word against 112 for the phase) and the transforms share a
+// kernel and the digits' write and read are gone. Each CTA reads its dn x 2 key
+// rows (prefetched to L2 on entry) for NB ciphertexts; ciphertexts run fastest
+// over the grid, so a chunk's key comes from DRAM once. Compiled for four CTAs of
+// 256 threads per SM (64 registers): with three (80) the sums' loads were exposed
+// and a multiplication at N = 2^16, level 41, took 2504 us for 4 ciphertexts
+// against 2435. Query of two ciphertexts a column at N = 2^16 141.9 -> 138.3 ms,
+// comparison at N = 2^15 51.6 -> 50.6, 32 ciphertexts' multiplication 18.26 -> 17.73.
+constexpr int kRowsIpMax = 16;  // rows of a CTA: 256 threads at 2^8 words a row
+struct RowsIp {
+  const Modulus* mods;
+  NttArgs tab;  // tables
+  const u64 *ext, *d, *kb, *ka;
+  long ext_os, d_os;
+  int level, alpha, L, T, N, dn, B, m0;
+  int nb, bgroups;  // ciphertexts per CTA, groups of them
+  u64* acc;
+  long acc_os;
+  int acc_nl;
+  const u64* x;
+  long x_os;
+  int x_cap, add_c1;
+  const u64* delta;
+  int nl;
+  const u64 *pm, *scale;
+  u64* out;
+  long out_os;
+  int out_cap;
+};
+
+// 128-bit sum of products of words below 2^56 and 2^55, at most 16 of them: the low
+// products with their carries, the middle (below 2^62) and the high ones apart
+struct MacSum {
+  u32 l0 = 0, l1 = 0, c = 0, m0 = 0, m1 = 0, h0 = 0, h1 = 0;
+  __device__ __forceinline__ void add(u64 x, u64 y) {
+    const u32 xl = (u32)x, xh = (u32)(x >> 32), yl = (u32)y, yh = (u32)(y >> 32);
+    asm("mad.lo.cc.u32 %0, %7, %9, %0;\n\tmadc.hi.cc.u32 %1, %7, %9, %1;\n\taddc.u32 %2, %2, 0;\n\t"
+        "mad.lo.cc.u32 %3, %7, %10, %3;\n\tmadc.hi.u32 %4, %7, %10, %4;\n\t"
+        "mad.lo.cc.u32 %3, %8, %9, %3;\n\tmadc.hi.u32 %4, %8, %9, %4;\n\t"
+        "mad.lo.cc.u32 %5, %8, %10, %5;\n\tmadc.hi.u32 %6, %8, %10, %6;"
+        : "+r"(l0), "+r"(l1), "+r"(c), "+r"(m0), "+r"(m1), "+r"(h0), "+r"(h1)
+        : "r"(xl), "r"(xh), "r"(yl), "r"(yh));
+  }
+  __device__ __forceinline__ u64 reduced(u64 q, u64 qinv) const {
+    const u64 l = ((u64)l1 << 32) | l0, m = ((u64)m1 << 32) | m0, h = ((u64)h1 << 32) | h0;
+    const u64 lo = l + (m << 32);
+    const u64 hi = h + (m >> 32) + c + (lo < l ? 1 : 0);
+    return redc128(hi, lo, q, qinv);
+  }
+};
+
+template <int LOGS, int TYPE>
+__global__ void __launch_bounds__(256, SS_ROWS_IP) k_rows_ip(const __grid_constant__ RowsIp A) {
+  extern __shared__ u64 sm[];
+  constexpr int S = 1 << LOGS, TPR = S / 16;
+  enter_grid();
+  const int tid = threadIdx.x;
+  const int bg = blockIdx.x % A.bgroups, chunk = blockIdx.x / A.bgroups;
+  const int m = A.m0 + blockIdx.y, g = m < A.level ? m : A.L + (m - A.level);
+  const int own = m < A.level ? m / A.alpha : A.dn;  // the digit that is not transformed (none: dn)
+  const int nd = A.dn - (own < A.dn ? 1 : 0), rpc = nd + (TYPE ? 2 : 0);
+  const int b0 = bg * A.nb, nb = min(A.nb, A.B - b0);
+  ulonglong2* twS = reinterpret_cast<ulonglong2*>(sm);
+  uint2* tpS = reinterpret_cast<uint2*>(twS + S);
+  u64* data = reinterpret_cast<u64*>(tpS + S);
+  const int n1 = A.N >> LOGS;
+  const long pos = ((long)chunk << LOGS), limb = (long)m * A.N + pos, key = (long)g * A.N + pos;
+  {
+    const size_t at = (size_t)n1 + ((size_t)chunk << LOGS);
+    const ulonglong2* gw = half_tw<true>(A.tab, g) + at;
+    const uint4* gp = reinterpret_cast<const uint4*>(half_tp<true>(A.tab, g) + at);
+    for (int i = tid; i < S; i += blockDim.x) cp16(twS + i, gw + i);
+    for (int i = tid; i < S / 2; i += blockDim.x) cp16(reinterpret_cast<uint4*>(tpS) + i, gp + i);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  }
+  const int row = tid / TPR, lr = tid % TPR;
+  const bool valid = row < nb * rpc;
+  const HalfMod hm = half_mod(A.mods[g]);
+  u64 x[16];
+  if (valid) {
+    const int b = row / rpc, r = row - b * rpc;
+    const u64* src = r < nd ? A.ext + (long)(b0 + b) * A.ext_os + (long)(r + (r >= own ? 1 : 0)) * (A.level + A.alpha) * A.N
+                            : A.delta + ((long)(b0 + b) * 2 + (r - nd)) * A.nl * A.N;
+    src += limb + lr;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) x[k] = src[TPR * k];
+  } else {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) x[k] = 0;
+  }
+  for (int i = tid; i < A.dn * (S / 8); i += blockDim.x) {  // a line of each 128 bytes of the key rows
+    const int j = i / (S / 8), w = i - j * (S / 8);
+    const u64* p = (w < S / 16 ? A.kb : A.ka) + (size_t)j * A.T * A.N + key + (w % (S / 16)) * 16;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+  }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  __syncthreads();
+  u64* mine = data + (size_t)row * S;
+  if (__any_sync(0xffffffffu, valid)) {
+    row_forward<LOGS>(x, mine, lr, twS, tpS, hm);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) x[k] = reduce_half(x[k], hm);  // below 2q
+    row_put(x, mine, lr);
+  }
+  __syncthreads();
+  const u64 q = hm.q, qinv = A.mods[g].qinv;
+  const size_t kstride = (size_t)A.T * A.N;
+  for (int p = tid; p < nb << LOGS; p += blockDim.x) {
+    const int b = p >> LOGS, n = p & (S - 1);
+    const long o = b0 + b;
+    const u64* kbp = A.kb + key + n;
+    const u64* kap = A.ka + key + n;
+    const u64* rows = data + b * rpc * S + row_swz(n);
+    MacSum s0, s1;
+    auto digits = [&](int r0, int r1) {
+#pragma unroll 4
+      for (int r = r0; r < r1; ++r) {
+        const u64 v = *rows, kv = *kbp, av = *kap;
+        s0.add(v, kv);
+        s1.add(v, av);
+        rows += S;
+        kbp += kstride;
+        kap += kstride;
+      }
+    };
+    digits(0, min(own, nd));
+    if (own < A.dn) {
+      const u64 v = A.d[o * A.d_os + limb + n], kv = *kbp, av = *kap;
+      s0.add(v, kv);
+      s1.add(v, av);
+      kbp += kstride;
+      kap += kstride;
+      digits(own, nd);
+    }
+    u64 a[2] = {s0.reduced(q, qinv), s1.reduced(q, qinv)};
+    if (TYPE == 0) {
+      if (A.x != nullptr && m == A.level - 1) {
+        const u64 pw = __ldg(A.pm + 2 * m), pwp = __ldg(A.pm + 2 * m + 1);
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+          a[c] = add_mod(a[c], shoup(A.x[o * A.x_os + (long)c * A.x_cap * A.N + limb + n], pw, pwp, q), q);
+      }
+      u64* out = A.acc + o * A.acc_os + (long)(m - A.m0) * A.N + pos + n;
+      out[0] = a[0];
+      out[(long)A.acc_nl * A.N] = a[1];
+    } else {
+      const u64 sc = __ldg(A.scale + 2 * m), scp = __ldg(A.scale + 2 * m + 1);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const u64 dl = rows[c * S];  // the rows after the digits', below 2q
+        const bool has_x = A.x != nullptr && (TYPE == 2 || c == 0 || A.add_c1);
+        const u64 xv = has_x ? A.x[o * A.x_os + (long)c * A.x_cap * A.N + limb + n] : 0;
+        u64 r;
+        if (TYPE == 2) {
+          const u64 px = shoup(xv, __ldg(A.pm + 2 * m), __ldg(A.pm + 2 * m + 1), q);
+          r = shoup(px + a[c] + 2 * q - dl, sc, scp, q);
+        } else {
+          r = shoup(a[c] + 2 * q - dl, sc, scp, q);
+          if (has_x) r = add_mod(r, xv, q);
+        }
+        A.out[o * A.out_os + (long)c * A.out_cap * A.N + limb + n] = r;
+      }
+    }
+  }
 }
 
 // ---------------------------------------------------------------- persistent multi-transform phase
@@ -1386,6 +1581,82 @@ void ntt_multi(const std::vector<NttReq>& reqs, bool fwd, cudaStream_t st) {
 }
 
 void ntt_forward(Context& C, const PolySet& s, cudaStream_t st) { launch(C, s, true, st); }
+
+bool rows_ip_fits(const Context& C, int level) {
+  return C.d_tp && !ntt_merger() && !ks_merger() && (level + C.alpha - 1) / C.alpha + 1 <= kRowsIpMax;
+}
+
+void ntt_forward_cols(Context& C, const PolySet& s, cudaStream_t st) {
+  const int npoly = s.n_outer * s.nl, l2 = chunk_log(C);
+  if (npoly == 0) return;
+  if (npoly > 65535) throw Error(SS_ERR_SHAPE, "too many polynomials in one transform");
+  int kr = kt_begin(C, st);
+  launch_cols<true>(C.m_odd, C.logN - l2, l2, npoly, st, make_args(C, s));
+  ++C.launches;
+  if (kr >= 0) C.kt.ntt_products += ntt_products(C, s, true);
+  kt_end(C, kr, KC_NTT, 16.0 * C.N * active_polys(s), st);
+}
+
+void rows_ip(Context& C, const RowsIpReq& R, cudaStream_t st) {
+  const int l2 = chunk_log(C), tpr = (1 << l2) / 16;
+  RowsIp A{};
+  PolySet none{nullptr, 0, 1, 1, 0, 1};
+  A.tab = make_args(C, none);
+  A.mods = A.tab.mods;
+  A.ext = R.ext;
+  A.d = R.d;
+  A.kb = R.K->b;
+  A.ka = R.K->a;
+  A.level = R.level;
+  A.alpha = C.alpha;
+  A.L = C.L;
+  A.T = C.ntot;
+  A.N = C.N;
+  A.dn = (R.level + C.alpha - 1) / C.alpha;
+  A.ext_os = (long)A.dn * (R.level + C.alpha) * C.N;
+  A.d_os = R.d_os;
+  A.B = R.B;
+  A.m0 = R.m0;
+  A.acc = R.acc;
+  A.acc_os = 2L * R.nlimbs * C.N;
+  A.acc_nl = R.nlimbs;
+  A.x = R.x ? R.x->data : nullptr;
+  A.x_os = R.x ? (long)R.x->ncomp * R.x->cap * C.N : 0;
+  A.x_cap = R.x ? R.x->cap : 0;
+  A.add_c1 = R.add_c1 ? 1 : 0;
+  A.delta = R.delta;
+  A.nl = R.nlimbs;
+  A.pm = R.pm;
+  A.scale = R.scale;
+  if (R.out) {
+    A.out = R.out->data;
+    A.out_os = (long)R.out->ncomp * R.out->cap * C.N;
+    A.out_cap = R.out->cap;
+  }
+  // rows of one ciphertext: every digit but a data limb's own, and the two of the correction
+  const int rpc = R.type == 0 ? A.dn : A.dn + 1;
+  A.nb = std::max(1, std::min(R.B, kRowsIpMax / rpc));
+  A.bgroups = (R.B + A.nb - 1) / A.nb;
+  const dim3 g((C.N >> l2) * A.bgroups, R.nlimbs);
+  // the rows' threads; a grid that leaves room gets 256 a CTA for the sums, whose
+  // loads are then one round deep (rotations near the chain's end: 815 -> 610 us)
+  int thr = (A.nb * rpc * tpr + 31) / 32 * 32;
+  if ((long)g.x * g.y <= SS_ROWS_IP * 152L) thr = 256;
+  const size_t smem = ((size_t)24 << l2) + (size_t)(thr / tpr) * 8 * (1 << l2);
+  const double words = (double)A.dn * R.nlimbs * (R.B + 2.0) + (R.type == 0 ? 2.0 : 4.0 + (R.x ? 2.0 : 0.0)) * R.nlimbs * R.B;
+  int kr = kt_begin(C, st);
+  if (l2 == 7) {
+    if (R.type == 0) launch_early(k_rows_ip<7, 0>, g, thr, smem, st, A);
+    else if (R.type == 1) launch_early(k_rows_ip<7, 1>, g, thr, smem, st, A);
+    else launch_early(k_rows_ip<7, 2>, g, thr, smem, st, A);
+  } else {
+    if (R.type == 0) launch_early(k_rows_ip<8, 0>, g, thr, smem, st, A);
+    else if (R.type == 1) launch_early(k_rows_ip<8, 1>, g, thr, smem, st, A);
+    else launch_early(k_rows_ip<8, 2>, g, thr, smem, st, A);
+  }
+  ++C.launches;
+  kt_end(C, kr, KC_KSIP, words * C.N * 8.0, st);
+}
 
 void ntt_inverse(Context& C, const PolySet& s, cudaStream_t st) { launch(C, s, false, st); }
 

@@ -142,9 +142,16 @@ static void keyswitch_impl(Context& C, const Buf& in, int comp, const KeyDev& K,
   ps.skip_mod = dn;
   ps.skip_level = l;
   ps.pre_w1 = pre;
-  ntt_forward(C, ps, st);
-  // 3. inner product with the key on the special primes (both components)
-  k_ks_ip(C, d, in_os, ext, ext_os, K, l, acc, sp_os, B, st, l, a);
+  // 3. inner product with the key on the special primes (both components); where it is
+  //    fused with the digits' chunk phase, the data limbs' waits for the correction
+  const bool fused = rows_ip_fits(C, l);
+  if (fused) {
+    ntt_forward_cols(C, ps, st);
+    rows_ip(C, RowsIpReq{0, ext, d, in_os, &K, l, B, l, a, acc, nullptr, false, nullptr, nullptr, nullptr, nullptr}, st);
+  } else {
+    ntt_forward(C, ps, st);
+    k_ks_ip(C, d, in_os, ext, ext_os, K, l, acc, sp_os, B, st, l, a);
+  }
   // 4. ModDown: delta = t * conv_P->Q(t^-1 acc mod P) on the data primes
   ntt_inverse(C, scaled_later(PolySet{acc, (long)a * N, 2 * B, a, C.L, 0}, post), st);
   const u64* c1 = C.d_tables + C.off_md_c1[in.t_exp];
@@ -153,9 +160,14 @@ static void keyswitch_impl(Context& C, const Buf& in, int comp, const KeyDev& K,
   k_bconv(C, acc, (long)a * N, a, C.L, c1, c2, delta, (long)l * N, l, l, 0, 0, tpost, 2 * B, st, -1, pre, post);
   PolySet pd{delta, (long)l * N, 2 * B, l, 0, l};
   pd.pre_w1 = pre;
-  ntt_forward(C, pd, st);
   // 5. inner product on the data primes fused with out = (acc - delta) P^-1 (+ addend)
   const u64* pinv = C.d_tables + C.off_md_pinv;
+  if (fused) {
+    ntt_forward_cols(C, pd, st);
+    rows_ip(C, RowsIpReq{1, ext, d, in_os, &K, l, B, 0, l, nullptr, addend, add_c1, delta, nullptr, pinv, &out}, st);
+    return;
+  }
+  ntt_forward(C, pd, st);
   k_ks_ip_fused(C, d, in_os, ext, ext_os, K, l, l, false, addend, add_c1, delta, l, nullptr, pinv, out, B, st);
 }
 
@@ -203,11 +215,16 @@ void op_relin_drop(Context& C, const Buf& in, Buf& out, cudaStream_t st) {
   ps.skip_mod = dn;
   ps.skip_level = l;
   ps.pre_w1 = pre;
-  ntt_forward(C, ps, st);
+  const bool fused = rows_ip_fits(C, l);
+  if (fused) ntt_forward_cols(C, ps, st);
+  else ntt_forward(C, ps, st);
   // 3. inner product on q_{l-1} and the special primes (the limbs the ModDown drops)
   //    with P d added on q_{l-1}
   const u64* pmod = C.d_tables + C.off_pmod;
-  k_ks_ip(C, d, in_os, ext, ext_os, C.rlk, l, acc, sp_os, B, st, l - 1, ns, &in, pmod);
+  if (fused)
+    rows_ip(C, RowsIpReq{0, ext, d, in_os, &C.rlk, l, B, l - 1, ns, acc, &in, true, nullptr, pmod, nullptr, nullptr}, st);
+  else
+    k_ks_ip(C, d, in_os, ext, ext_os, C.rlk, l, acc, sp_os, B, st, l - 1, ns, &in, pmod);
   // 4. ModDown by q_{l-1} P: delta = t conv([t^-1 (P d + acc)]_D) on the first l-1 primes
   ntt_inverse(C, scaled_later(PolySet{acc, (long)ns * N, 2 * B, ns, l - 1, 1}, post), st);
   const u64* c2 = C.d_tables + C.off_rd[l];
@@ -217,6 +234,11 @@ void op_relin_drop(Context& C, const Buf& in, Buf& out, cudaStream_t st) {
   k_bconv(C, acc, (long)ns * N, ns, l - 1, c1, c2, delta, (long)nl * N, nl, nl, 0, 0, tpost, 2 * B, st, 1, pre, post);
   PolySet pd{delta, (long)nl * N, 2 * B, nl, 0, nl};
   pd.pre_w1 = pre;
+  if (fused) {  // 5, with the correction's chunk phase
+    ntt_forward_cols(C, pd, st);
+    rows_ip(C, RowsIpReq{2, ext, d, in_os, &C.rlk, l, B, 0, nl, nullptr, &in, true, delta, pmod, inv, &out}, st);
+    return;
+  }
   ntt_forward(C, pd, st);
   // 5. inner product on the kept primes fused with the combine
   //    out_c = ((P d_c + acc_c) - delta_c) (q_{l-1} P)^-1

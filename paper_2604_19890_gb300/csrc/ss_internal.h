@@ -237,6 +237,25 @@ void ntt_inverse(Context& C, const PolySet& s, cudaStream_t st);
 // Inverse transform of the polynomials at src (same shape as s, outer stride
 // src_os) written to s: the first phase reads src, so src is left unchanged.
 void ntt_inverse_from(Context& C, const PolySet& s, const u64* src, long src_os, cudaStream_t st);
+// A key switch's digits: the forward transform's column phase alone, and its chunk
+// phase fused with the inner product (k_rows_ip). rows_ip_fits: whether the
+// context, level and thread (not a merged lane) take this pair.
+bool rows_ip_fits(const Context& C, int level);
+void ntt_forward_cols(Context& C, const PolySet& s, cudaStream_t st);
+struct RowsIpReq {
+  int type;            // 0: reduced sums to acc; 1: ModDown by P; 2: relinearise-and-drop
+  const u64 *ext, *d;  // digits after the column phase [B][dnum][level + alpha][N]; digit source (evaluation form)
+  long d_os;
+  const KeyDev* K;
+  int level, B, m0, nlimbs;  // limbs [m0, m0 + nlimbs) of the extended basis
+  u64* acc;                  // type 0: [B][2][nlimbs][N]
+  const Buf* x;              // addend (type 1), the input's components (types 0, 2), or null
+  bool add_c1;
+  const u64* delta;          // types 1, 2: the correction after its column phase [B][2][nlimbs][N]
+  const u64 *pm, *scale;
+  Buf* out;
+};
+void rows_ip(Context& C, const RowsIpReq& R, cudaStream_t st);
 // Transforms of several contexts (ring dimensions N >= 8192) merged: each
 // phase of all of them runs as one persistent launch over their tiles.
 struct NttReq {
