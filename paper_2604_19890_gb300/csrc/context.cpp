@@ -644,7 +644,7 @@ void build_context(Context& C, const ss_params& prm) {
   }
   upload((void**)&C.d_mod, md.data(), sizeof(ModDesc) * T);
 
-  std::vector<u64> r64(4 * T, 0), fold_w1(T, 1);  // fold_w1: the forward node-1 twiddle of X^N + 1
+  std::vector<u64> r64(kR64 * T, 0), fold_w1(T, 1);  // fold_w1: the forward node-1 twiddle of X^N + 1
   // twiddles: psi^brv(i) and psi^-brv(i) with Shoup companions (m = 2N; m = 3N below)
   {
     // transforms of N >= 8192 multiply by halves where the primes leave nine spare bits
@@ -658,7 +658,11 @@ void build_context(Context& C, const ss_params& prm) {
     std::vector<u64> split(C.m_odd == 5 ? (size_t)T * 24 : 0);
     for (int i = 0; i < T; ++i) {
       u64 q = C.primes[i], ps = C.psi[i], pi = nt::inv(ps, q);
-      r64[4 * i] = (UINT64_MAX % q + 1) % q;  // 2^64 mod q
+      u64* rr = &r64[(size_t)kR64 * i];
+      rr[0] = (UINT64_MAX % q + 1) % q;  // 2^64 mod q
+      rr[4] = (1ULL << 32) % q;
+      rr[6] = (1ULL << 62) % q;
+      rr[8] = (1ULL << 61) % q;
       u64* o = &tw[(size_t)i * 4 * slots];
       auto put = [&](int node, u64 f, u64 bk) {
         const size_t k = halves && node > 0 ? slot[node] : node;
@@ -746,12 +750,12 @@ void build_context(Context& C, const ss_params& prm) {
           int rk = nt::brv(k, C.logN);
           put(k, fw[rk], bw[rk]);
         }
-        // 2^64 times the forward node-1 twiddle psi^bitrev(1) = psi^(N/2)
+        // times the forward node-1 twiddle psi^bitrev(1) = psi^(N/2)
         fold_w1[i] = fw[N / 2];
-        r64[4 * i + 1] = nt::mul(r64[4 * i], fw[N / 2], q);
+        for (int e : {0, 4, 6, 8}) rr[e + 1] = nt::mul(rr[e], fw[N / 2], q);
         // 2^64 N^-1 and 2^64 N^-1 psi^(-N/2): the inverse's last-stage factors of the lower and upper half
-        r64[4 * i + 2] = nt::mul(r64[4 * i], ni, q);
-        r64[4 * i + 3] = nt::mul(r64[4 * i + 2], bw[N / 2], q);
+        rr[2] = nt::mul(rr[0], ni, q);
+        rr[3] = nt::mul(rr[2], bw[N / 2], q);
         // N^-1 times the last inverse stage's twiddle psi^-bitrev(1) = psi^(-N/2)
         const u64 wni = nt::mul(ni, bw[N / 2], q);
         ninv[6 * i + 2] = wni;
@@ -896,7 +900,7 @@ void build_context(Context& C, const ss_params& prm) {
         for (int s = 0; s < cnt; ++s) {
           const u64 qs = C.primes[j * al + s];
           // X^N + 1: 2^64 N^-1, 2^64 N^-1 psi^(-N/2) (d_r64), the inverse's last stage; other rings 2^64
-          row[s] = nt::mul(c1[2 * s], r64[4 * (j * al + s) + (C.m_odd == 1 ? 2 + u : 0)], qs);
+          row[s] = nt::mul(c1[2 * s], r64[(size_t)kR64 * (j * al + s) + (C.m_odd == 1 ? 2 + u : 0)], qs);
           for (int g = 0; g < T; ++g) {
             const u64 q = C.primes[g];
             const u64 w = nt::mul(c2[(size_t)s * T + g], u && C.m_odd == 1 ? fold_w1[g] : 1, q);

@@ -33,9 +33,6 @@ constexpr int TPB = 256;
 #ifndef SS_KSIP_OB
 #define SS_KSIP_OB 2  // ciphertexts per thread in the key-switch inner product
 #endif
-#ifndef SS_BCONV_V
-#define SS_BCONV_V 2  // coefficients per thread in base conversion (1 to 4 sources)
-#endif
 #ifndef SS_KSIP_V
 #define SS_KSIP_V 2  // coefficients per thread in the key-switch inner product
 #endif
@@ -199,81 +196,115 @@ __global__ void k_tensor_impl(const u64* a, const u64* b, u64* out, int N, int l
 }
 
 // ---------------------------------------------------------------- base conversion
+// r_i = 2^-32 sum_s (yl_s,i c_2s + yh_s,i c_(2s+1)) mod q by one Montgomery step; the
+// low products' sum is below 2^64. qi = -q^-1 mod 2^32.
+template <int NS, int V>
+__device__ __forceinline__ void sum_halves(const u32 (&yl)[NS][V], const u32 (&yh)[NS][V], const u64* c, u64 q, u32 qi,
+                                           u64 (&r)[V]) {
+  u32 a0[V], a1[V], h0[V], h1[V];
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    const u64 c0 = c[2 * s], c1 = c[2 * s + 1];
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+      if (s == 0) a0[i] = a1[i] = h0[i] = h1[i] = 0;
+      mac_pair(a0[i], a1[i], yl[s][i], (u32)c0);
+      mac_pair(a0[i], a1[i], yh[s][i], (u32)c1);
+      mac_pair(h0[i], h1[i], yl[s][i], (u32)(c0 >> 32));
+      mac_pair(h0[i], h1[i], yh[s][i], (u32)(c1 >> 32));
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < V; ++i) {
+    const u32 m = a0[i] * qi;
+    u32 r0, r1;
+    asm("{\n\t"
+        ".reg .u32 t0, t1, c, g0, g1;\n\t"
+        "mad.lo.cc.u32 t0, %2, %3, %5;\n\t"
+        "madc.hi.cc.u32 t1, %2, %3, %6;\n\t"
+        "addc.u32 c, 0, 0;\n\t"
+        "mad.lo.cc.u32 g0, %2, %4, %7;\n\t"
+        "madc.hi.u32 g1, %2, %4, %8;\n\t"
+        "add.cc.u32 %0, g0, t1;\n\t"
+        "addc.u32 %1, g1, c;\n\t"
+        "}"
+        : "=r"(r0), "=r"(r1)
+        : "r"(m), "r"((u32)q), "r"((u32)(q >> 32)), "r"(a0[i]), "r"(a1[i]), "r"(h0[i]), "r"(h1[i]));
+    r[i] = ((u64)r1 << 32) | r0;
+  }
+}
+
 // dst limb m (global prime g(m) = m < nq ? m : L + m - nq), m outside
 // [skip_lo, skip_hi):  sum_s [src_s * c1_s]_{q_s} * c2[s][g(m)]  (mod q_g), then
 // times post[g] when post != null. Source s lives on prime sp0 + s (s < nsq)
-// or L + s - nsq. Per block, each target's modulus, its Montgomery inverse and
-// the constants c2[s][g] * post[g] * 2^64 mod q_g are staged once in shared
-// memory (row m: q, -q^-1 mod 2^64, c2'[0..ns)); every output is then a
-// 128-bit sum of ns products and one Montgomery reduction, which removes the
-// 2^64 and leaves the post factor applied. The sum stays below ns q_s q_g <
-// q_g 2^64 (primes below 2^58, ns <= 64), as the reduction needs.
-// V = 2: two consecutive coefficients per thread (16-byte accesses, the
-// staged constants read once for both).
-// tw != null (ModUp on the ring X^N + 1): outputs of the upper half
-// (coefficients n >= N/2) also carry the forward transform's node-1 twiddle
-// w_1 = psi^(N/2) of their prime, so the transform skips its first stage's
-// product (PolySet::pre_w1). A block's V*blockDim coefficients lie in one
-// half (the host checks that they divide N/2), so a block of the upper half
-// stages c2'[s] w_1 2^64 instead (the factor 2^64 w_1 mod q comes from the
-// per-prime table r64 beside 2^64 mod q; no product per output).
+// or L + s - nsq. Words come out below 3q, as the forward transforms take them
+// (below 4q). NS <= 4 sources, halves of y_s and one Montgomery step by 2^32 as
+// in k_modup; SPLIT low bits keep the low products' sum below 2^64 also for
+// 58-bit primes (8 (2^29 - 1)(2^32 - 1) for NS = 4). Per block, each target's
+// modulus, -q^-1 mod 2^64 and the pairs (c2 post 2^32, c2 post 2^(32+SPLIT)) mod
+// q_g are staged once in shared memory (row m: q, -q^-1, the pairs), one thread a
+// pair. (128-bit sums and a Montgomery step by 2^64 kept the multiply pipe 81 %
+// busy at 80 us for 4 sources, 40 targets, 8 polynomials of 2^16 words.)
+// pre (ring X^N + 1): outputs of the upper half (coefficients n >= N/2) also
+// carry the forward transform's node-1 twiddle w_1 = psi^(N/2) of their prime,
+// so the transform skips its first stage's product (PolySet::pre_w1): a block's
+// coefficients lie in one half (the host checks that they divide N/2), and an
+// upper-half block takes its factors from the table's w_1 entries.
 // dscale (sources from an inverse transform with PolySet::post_scale): the
 // source words still lack N^-1 (lower half) or N^-1 psi^(-N/2) (upper half),
-// and may be up to 4q; the first step then uses c1_s times that factor in
+// and may be any 64-bit words; the first step then uses c1_s times that factor in
 // Montgomery form (staged per block after the targets' rows) and a Montgomery
-// reduction in place of the Shoup product, which accepts any 64-bit word.
-template <int NS, int V>
-__global__ void __launch_bounds__(256) k_bconv_impl(const u64* src, long src_os, int ns, int sp0, int nsq,
+// reduction in place of the Shoup product.
+template <int NS>
+__global__ void __launch_bounds__(256) k_bconv_impl(const u64* src, long src_os, int sp0, int nsq,
                                                     const u64* __restrict__ c1, const u64* __restrict__ c2, int T,
                                                     u64* __restrict__ dst, long dst_os, int nd, int nq, int L,
                                                     int skip_lo, int skip_hi, const u64* __restrict__ post, int N,
                                                     const ModDesc* mods, const u64* __restrict__ r64, int pre,
                                                     int dscale) {
   enter_grid();
+  constexpr int V = 2, SPLIT = NS < 4 ? 30 : 29, W = 2 + 2 * NS;
   extern __shared__ u64 sh[];
-  const int ns_ = NS > 0 ? NS : ns;
-  const int W = 2 + ns_;
   const int half = 2 * V * blockIdx.x * blockDim.x >= N ? 1 : 0;  // block-uniform
   const int upper = pre ? half : 0;
   if (dscale)
-    for (int s = threadIdx.x; s < ns_; s += blockDim.x) {
+    for (int s = threadIdx.x; s < NS; s += blockDim.x) {
       const int gs = s < nsq ? sp0 + s : L + (s - nsq);
-      sh[nd * W + s] = mul_mod(__ldg(c1 + 2 * s), __ldg(r64 + 4 * gs + 2 + half), MOD(mods, gs));
+      sh[nd * W + s] = mul_mod(__ldg(c1 + 2 * s), __ldg(r64 + kR64 * gs + 2 + half), MOD(mods, gs));
     }
-  for (int m = threadIdx.x; m < nd; m += blockDim.x) {
+  for (int i = threadIdx.x; i < nd * NS; i += blockDim.x) {
+    const int m = i / NS, s = i - m * NS;
     const int g = m < nq ? m : L + (m - nq);
     const Modulus& md = MOD(mods, g);
     u64* e = sh + m * W;
-    e[0] = md.q;
-    e[1] = md.qinv;
-    const u64 R = __ldg(r64 + 4 * g + upper);  // 2^64 (times w_1) mod q
-    for (int s = 0; s < ns_; ++s) {
-      u64 v = c2[(long)s * T + g];
-      if (post) v = shoup(v, post[2 * g], post[2 * g + 1], md.q);
-      e[2 + s] = mul_mod(v, R, md);
+    if (s == 0) {
+      e[0] = md.q;
+      e[1] = md.qinv;
     }
+    u64 v = c2[(long)s * T + g];
+    if (post) v = shoup(v, post[2 * g], post[2 * g + 1], md.q);
+    const u64* f = r64 + kR64 * g + upper;
+    e[2 + 2 * s] = mul_mod(v, __ldg(f + 4), md);
+    e[3 + 2 * s] = mul_mod(v, __ldg(f + (NS < 4 ? 6 : 8)), md);
   }
   __syncthreads();
   const int o = blockIdx.y;
   const int n = V * (blockIdx.x * blockDim.x + threadIdx.x);
   if (n >= N) return;
-  constexpr int MAXS = NS > 0 ? NS : 64;
-  u64 y[V][MAXS];
+  u32 yl[NS][V], yh[NS][V];
 #pragma unroll
-  for (int s = 0; s < MAXS; ++s) {
-    if (s < ns_) {
-      const int gs = s < nsq ? sp0 + s : L + (s - nsq);
-      const Modulus& ms = MOD(mods, gs);
-      u64 v[V];
-      ldv<V>(src + o * src_os + (long)s * N + n, v);
-      if (dscale) {
-        const u64 cm = sh[nd * W + s];
+  for (int s = 0; s < NS; ++s) {
+    const int gs = s < nsq ? sp0 + s : L + (s - nsq);
+    const Modulus& ms = MOD(mods, gs);
+    u64 v[V];
+    ldv<V>(src + o * src_os + (long)s * N + n, v);
+    const u64 cm = dscale ? sh[nd * W + s] : 0;
 #pragma unroll
-        for (int i = 0; i < V; ++i) y[i][s] = redc128(mulhi64(v[i], cm), v[i] * cm, ms.q, ms.qinv);
-      } else {
-#pragma unroll
-        for (int i = 0; i < V; ++i) y[i][s] = shoup(v[i], c1[2 * s], c1[2 * s + 1], ms.q);
-      }
+    for (int i = 0; i < V; ++i) {
+      const u64 y = dscale ? redc128(mulhi64(v[i], cm), v[i] * cm, ms.q, ms.qinv)
+                           : shoup(v[i], c1[2 * s], c1[2 * s + 1], ms.q);
+      yl[s][i] = (u32)y & ((1u << SPLIT) - 1);
+      yh[s][i] = (u32)(y >> SPLIT);
     }
   }
   u64* out = dst + o * dst_os + n;
@@ -281,21 +312,8 @@ __global__ void __launch_bounds__(256) k_bconv_impl(const u64* src, long src_os,
     const int m0 = part == 0 ? 0 : skip_hi, m1 = part == 0 ? min(skip_lo, nd) : nd;
     for (int m = m0; m < m1; ++m) {
       const u64* e = sh + m * W;
-      Acc128 acc[V];
-#pragma unroll
-      for (int v = 0; v < V; ++v) acc[v].zero();
-#pragma unroll
-      for (int s = 0; s < MAXS; ++s) {
-        if (s < ns_) {
-          const u64 cs = e[2 + s];
-#pragma unroll
-          for (int v = 0; v < V; ++v) acc[v].mac_wide(y[v][s], cs);
-        }
-      }
-      const u64 qm = e[0], qi = e[1];
       u64 r[V];
-#pragma unroll
-      for (int i = 0; i < V; ++i) r[i] = redc128(acc[i].hi, acc[i].lo, qm, qi);
+      sum_halves<NS, V>(yl, yh, e + 2, e[0], (u32)e[1], r);
       stv<V>(out + (long)m * N, r);
     }
   }
@@ -323,7 +341,7 @@ __global__ void __launch_bounds__(256) k_bconv_many_impl(const u64* src, long sr
   if (dscale)
     for (int s = threadIdx.x; s < ns; s += blockDim.x) {
       const int gs = s < nsq ? sp0 + s : L + (s - nsq);
-      sh[nd * W + s] = mul_mod(__ldg(c1 + 2 * s), __ldg(r64 + 4 * gs + 2 + half), MOD(mods, gs));
+      sh[nd * W + s] = mul_mod(__ldg(c1 + 2 * s), __ldg(r64 + kR64 * gs + 2 + half), MOD(mods, gs));
     }
   for (int m = threadIdx.x; m < nd; m += blockDim.x) {
     const int g = m < nq ? m : L + (m - nq);
@@ -331,7 +349,7 @@ __global__ void __launch_bounds__(256) k_bconv_many_impl(const u64* src, long sr
     u64* e = sh + m * W;
     e[0] = md.q;
     e[1] = md.qinv;
-    const u64 R = __ldg(r64 + 4 * g + upper);  // 2^64 (times w_1) mod q
+    const u64 R = __ldg(r64 + kR64 * g + upper);  // 2^64 (times w_1) mod q
     for (int s = 0; s < ns; ++s) {
       u64 v = c2[(long)s * T + g];
       if (post) v = shoup(v, post[2 * g], post[2 * g + 1], md.q);
@@ -456,40 +474,8 @@ __global__ void __launch_bounds__(256) k_modup_impl(const ModupArgs A) {
   u64* out = A.dst + ((long)b * A.dn + j) * nx * A.N + n;
   for (int t = t0; t < t1; ++t) {
     const u64* e = sh + (t - t0) * W;
-    u32 a0[V], a1[V], h0[V], h1[V];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      const u64 c0 = e[2 * s], c1 = e[2 * s + 1];
-#pragma unroll
-      for (int i = 0; i < V; ++i) {
-        if (s == 0) a0[i] = a1[i] = h0[i] = h1[i] = 0;
-        mac_pair(a0[i], a1[i], yl[s][i], (u32)c0);
-        mac_pair(a0[i], a1[i], yh[s][i], (u32)c1);
-        mac_pair(h0[i], h1[i], yl[s][i], (u32)(c0 >> 32));
-        mac_pair(h0[i], h1[i], yh[s][i], (u32)(c1 >> 32));
-      }
-    }
-    const u64 q = e[2 * NS];
-    const u32 qi = (u32)e[2 * NS + 1];
     u64 r[V];
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-      const u32 m = a0[i] * qi;
-      u32 r0, r1;
-      asm("{\n\t"
-          ".reg .u32 t0, t1, c, g0, g1;\n\t"
-          "mad.lo.cc.u32 t0, %2, %3, %5;\n\t"
-          "madc.hi.cc.u32 t1, %2, %3, %6;\n\t"
-          "addc.u32 c, 0, 0;\n\t"
-          "mad.lo.cc.u32 g0, %2, %4, %7;\n\t"
-          "madc.hi.u32 g1, %2, %4, %8;\n\t"
-          "add.cc.u32 %0, g0, t1;\n\t"
-          "addc.u32 %1, g1, c;\n\t"
-          "}"
-          : "=r"(r0), "=r"(r1)
-          : "r"(m), "r"((u32)q), "r"((u32)(q >> 32)), "r"(a0[i]), "r"(a1[i]), "r"(h0[i]), "r"(h1[i]));
-      r[i] = ((u64)r1 << 32) | r0;
-    }
+    sum_halves<NS, V>(yl, yh, e, e[2 * NS], (u32)e[2 * NS + 1], r);
     stv<V>(out + (long)(t < lo ? t : t + cnt) * A.N, r);
   }
 }
@@ -1395,23 +1381,20 @@ void k_bconv(Context& C, const u64* src, long src_os, int ns, int sp0, const u64
   if (nsq < 0) nsq = ns;  // every source is the data or special prime sp0 + s
   dim3 g = grid_for(C.N, n_outer);
   if (ns < 1 || ns > 64) throw Error(SS_ERR_PARAM, "base conversion from 1..64 primes");
-  static_assert(SS_BCONV_V == 2, "both base-conversion kernels cover 2 * 256 coefficients per block");
-  if ((pre_w1 || post_scale) && (C.m_odd != 1 || (C.N / 2) % (SS_BCONV_V * TPB) != 0))
+  if ((pre_w1 || post_scale) && (C.m_odd != 1 || (C.N / 2) % (2 * TPB) != 0))
     throw Error(SS_ERR_PARAM, "twiddle folding needs the ring X^N + 1 and N >= 1024");
   if (skip_hi <= skip_lo) skip_lo = skip_hi = nd;
   const int pre = pre_w1 ? 1 : 0, dscale = post_scale ? 1 : 0;
-  size_t smem = (size_t)(nd * (2 + ns) + dscale * ns) * 8;
+  size_t smem = (size_t)(nd * (2 + (ns <= 4 ? 2 : 1) * ns) + dscale * ns) * 8;
   if (smem > 48 * 1024) throw Error(SS_ERR_PARAM, "base conversion tables exceed 48 KiB of shared memory");
   int kr_ = kt_begin(C, st);
-#define SS_BCONV(NSV, VV)                                                                                        \
-  launch_early(k_bconv_impl<NSV, VV>, dim3((g.x + VV - 1) / VV, g.y), TPB, smem, st,                                        \
-      src, src_os, ns, sp0, nsq, c1, c2, C.ntot, dst, dst_os, nd, nq, C.L, skip_lo, skip_hi, post, C.N, C.d_mod,     \
-      C.d_r64, pre, dscale)
+#define SS_BCONV(NSV)                                                                                              \
+  case NSV:                                                                                                        \
+    launch_early(k_bconv_impl<NSV>, dim3((g.x + 1) / 2, g.y), TPB, smem, st, src, src_os, sp0, nsq, c1, c2, C.ntot, \
+                 dst, dst_os, nd, nq, C.L, skip_lo, skip_hi, post, C.N, C.d_mod, C.d_r64, pre, dscale);            \
+    break;
   switch (ns) {
-    case 1: SS_BCONV(1, SS_BCONV_V); break;
-    case 2: SS_BCONV(2, SS_BCONV_V); break;
-    case 3: SS_BCONV(3, SS_BCONV_V); break;
-    case 4: SS_BCONV(4, SS_BCONV_V); break;
+    SS_BCONV(1) SS_BCONV(2) SS_BCONV(3) SS_BCONV(4)
     default:
       launch_early(k_bconv_many_impl<4, 2>, dim3((g.x + 1) / 2, g.y), TPB, smem, st, 
           src, src_os, ns, sp0, nsq, c1, c2, C.ntot, dst, dst_os, nd, nq, C.L, skip_lo, skip_hi, post, C.N, C.d_mod,

@@ -713,7 +713,7 @@ __device__ __forceinline__ void half_settle(u64 (&x)[16], int ns, const HalfMod&
 template <int CL>
 __device__ __forceinline__ int col_swz(int lin) {
   // eight columns: rows 16 apart would share banks; odd groups of 16 rows swap row pairs
-  return CL == 3 ? lin ^ (((lin >> 7) & 1) << 3) : lin;
+  return CL == 2 ? lin ^ (((lin >> 6) & 3) << 2) : CL == 3 ? lin ^ (((lin >> 7) & 1) << 3) : lin;
 }
 
 template <bool FWD, int LOGS, int LOG2N, int CL, int RING>
@@ -842,14 +842,17 @@ __device__ __forceinline__ void ntt16_cols(const NttArgs& A, int tile, int poly)
   }
 }
 
-constexpr int kColTile = 11;  // log2 words of a column tile: 128 threads
+#ifndef SS_COLTILE
+#define SS_COLTILE 11
+#endif
+constexpr int kColTile = SS_COLTILE, kColThr = (1 << kColTile) / 16;  // log2 words of a column tile, its threads
 template <int LOGS, int CL>
 constexpr size_t col_smem() {
   return ((size_t)24 << LOGS) + ((size_t)8 << (LOGS + CL));
 }
 
 template <bool FWD, int LOGS, int LOG2N, int CL, int RING>
-__global__ void __launch_bounds__(128, FWD ? SS_COLS_F : SS_COLS_I) k_ntt16_cols(NttArgs A) {
+__global__ void __launch_bounds__(kColThr, (FWD ? SS_COLS_F : SS_COLS_I) * 128 / kColThr) k_ntt16_cols(NttArgs A) {
   enter_grid();
   ntt16_cols<FWD, LOGS, LOG2N, CL, RING>(A, blockIdx.x, blockIdx.y);
 }
@@ -1236,7 +1239,7 @@ __device__ __noinline__ void ntt16_rows_fn(const NttArgs& A, const RowPlan& R, i
 }
 
 template <bool FWD, bool COLS, bool SRC>
-__global__ void __launch_bounds__(128, 6) k_ntt16_multi(const __grid_constant__ NttMulti M) {
+__global__ void __launch_bounds__(COLS ? kColThr : 128, COLS ? 6 * 128 / kColThr : 6) k_ntt16_multi(const __grid_constant__ NttMulti M) {
   for (int t = blockIdx.x; t < M.total; t += gridDim.x) {
     int j = 0;
     while (j + 1 < M.njobs && t >= M.j[j + 1].start) ++j;
@@ -1273,7 +1276,7 @@ __global__ void __launch_bounds__(128, 6) k_ntt16_multi(const __grid_constant__ 
 template <bool FWD, int LOGS, int LOG2N, int RING>
 void launch_cols_as(int npoly, cudaStream_t st, const NttArgs& A) {
   constexpr int CL = kColTile - LOGS;
-  launch_early(k_ntt16_cols<FWD, LOGS, LOG2N, CL, RING>, dim3(1 << (LOG2N - CL), npoly), 128, col_smem<LOGS, CL>(), st, A);
+  launch_early(k_ntt16_cols<FWD, LOGS, LOG2N, CL, RING>, dim3(1 << (LOG2N - CL), npoly), kColThr, col_smem<LOGS, CL>(), st, A);
 }
 template <bool FWD>
 void launch_cols(int ring, int logS, int log2n, int npoly, cudaStream_t st, const NttArgs& A) {
@@ -1568,11 +1571,11 @@ void ntt_multi(const std::vector<NttReq>& reqs, bool fwd, cudaStream_t st) {
     Context& C0 = *reqs[b0].C;
     int kr = kt_begin(C0, st);
     if (fwd) {
-      launch_multi<true, true, false>(P1, 128, smem_cols, st);
+      launch_multi<true, true, false>(P1, kColThr, smem_cols, st);
       launch_multi<true, false, false>(P2, thr, smem_rows, st);
     } else {
       launch_multi<false, false, true>(P1, thr, smem_rows, st);
-      launch_multi<false, true, false>(P2, 128, smem_cols, st);
+      launch_multi<false, true, false>(P2, kColThr, smem_cols, st);
     }
     C0.launches += 2;
     if (kr >= 0) C0.kt.ntt_products += prods;

@@ -47,6 +47,8 @@ std::vector<i64> g_coeffs_reduced(int p, int e);  // equivalent, least sum of |c
 std::vector<i64> flt_coeffs(int p);       // centred mod p
 }  // namespace nt
 
+// words per prime of Context::d_r64
+constexpr int kR64 = 10;
 // words of one row of Context::d_modup
 __host__ __device__ inline size_t modup_row_words(int T, int alpha) { return (size_t)alpha * (1 + 2 * (size_t)T); }
 
@@ -139,8 +141,9 @@ struct Context {
                                       //   halves: per prime and direction ntt_tw_slots pairs (w, 2^32 w mod q)
   u32* d_tp = nullptr;                // products by halves (N >= 8192, primes below 2^55): for each pair of d_tw the
                                       //   two half-quotients floor(w 2^31 / q); else null
-  u64* d_r64 = nullptr;               // [ntot][4] 2^64 mod q; X^N + 1: 2^64 psi^(N/2) (forward node 1),
-                                      //   2^64 N^-1, 2^64 N^-1 psi^(-N/2) (the inverse's last stage)
+  u64* d_r64 = nullptr;               // [ntot][kR64] mod q: 2^64, 2^64 w; 2^64 N^-1, 2^64 N^-1 psi^(-N/2) (the inverse's
+                                      //   last stage); 2^32, 2^32 w; 2^62, 2^62 w; 2^61, 2^61 w, with w the forward
+                                      //   node-1 twiddle psi^(N/2) (entries with w, N^-1: X^N + 1 only)
   u64* d_ninv = nullptr;              // [ntot][6] N^{-1}, shoup, N^{-1} psi^{-N/2} (m = 3N: 2 c), shoup, (m = 3N: c =
                                       //   (2 rho - 1)^{-1} N^{-1}), shoup
   u64* d_split = nullptr;             // m = 5N/2: [ntot][12][2] four-way split constants (forward 5, inverse 7)

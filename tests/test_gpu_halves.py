@@ -73,6 +73,27 @@ def test_multiplication_with_ragged_digits(ring, bits, count, level):
         assert (w[i] == o.mul(oa[i], ob[i]).words()).all()
 
 
+@pytest.mark.parametrize("level", [14, 15, 16, 17])
+@pytest.mark.parametrize("count", [1, 2])
+def test_digit_counts_around_the_fused_limit(count, level):
+    """Key switches of one-prime digits where the fused inner product's rows fill a CTA (15 digits and the
+    correction's two less one) and where they no longer fit, through a relinearisation and a multiplication."""
+    import paper_2604_19890_gb300 as ssg
+    kw = dict(logN=13, L=17, alpha=1, bits=50, p=17, r=1, h=8, seed=29, m_odd=0)
+    g, o = ssg.Context(nmax=0, **kw), O.Oracle(**kw)
+    g.keygen([])
+    o.keygen([])
+    rng = np.random.default_rng(level)
+    vals = rng.integers(0, g.t, (count, g.slots))
+    a = g.encrypt(np.stack([g.encode(v) for v in vals]), 3)
+    oa = [o.encrypt(o.encode(v), 3 + i) for i, v in enumerate(vals)]
+    if level < 17:
+        a, oa = g.modswitch(a, 17 - level), [o.modswitch(x, 17 - level) for x in oa]
+    rel, mul = g.relin(g.mul(a, a)).words(), g.mul_relin(a, a).words()
+    assert (rel[-1] == o.relin(o.tensor(oa[-1], oa[-1])).words()).all()
+    assert (mul[0] == o.mul(oa[0], oa[0]).words()).all()
+
+
 @pytest.mark.parametrize("nin,nout", [(1, 1), (2, 16), (7, 3), (15, 8), (16, 16)])
 @pytest.mark.parametrize("bits,logN", [(36, 9), (55, 13), (58, 8)])
 def test_small_coefficient_combinations(bits, logN, nin, nout):
