@@ -50,6 +50,9 @@ constexpr int TILE = 4096;  // words per CTA tile (32 KiB of shared memory)
 #ifndef SS_COLS_I
 #define SS_COLS_I 7
 #endif
+#ifndef SS_COLS_BIG
+#define SS_COLS_BIG 4  // of 256 threads
+#endif
 #ifndef SS_ROWS_F
 #define SS_ROWS_F 7
 #endif
@@ -713,7 +716,7 @@ __device__ __forceinline__ void half_settle(u64 (&x)[16], int ns, const HalfMod&
 template <int CL>
 __device__ __forceinline__ int col_swz(int lin) {
   // eight columns: rows 16 apart would share banks; odd groups of 16 rows swap row pairs
-  return CL == 2 ? lin ^ (((lin >> 6) & 3) << 2) : CL == 3 ? lin ^ (((lin >> 7) & 1) << 3) : lin;
+  return CL == 3 ? lin ^ (((lin >> 7) & 1) << 3) : lin;
 }
 
 template <bool FWD, int LOGS, int LOG2N, int CL, int RING>
@@ -842,17 +845,21 @@ __device__ __forceinline__ void ntt16_cols(const NttArgs& A, int tile, int poly)
   }
 }
 
-#ifndef SS_COLTILE
-#define SS_COLTILE 11
-#endif
-constexpr int kColTile = SS_COLTILE, kColThr = (1 << kColTile) / 16;  // log2 words of a column tile, its threads
+// log2 words of a column tile: small (128 threads) or large (256 threads, twice the
+// columns: 128-byte rows at 2^8 words a column, half the twiddle copies). A
+// multiplication at N = 2^16, level 41, of 1, 4 and 32 ciphertexts takes 666, 2411
+// and 17491 us with the small tile and 652, 2337 and 17231 with the large one (a
+// tile of 2^10 words: 702, 2562, 19986), so the large one runs wherever its
+// tiles fill the GPU twice; below that the small one spreads the work wider.
+constexpr int kColTile = 11, kColTileBig = 12;
 template <int LOGS, int CL>
 constexpr size_t col_smem() {
   return ((size_t)24 << LOGS) + ((size_t)8 << (LOGS + CL));
 }
 
 template <bool FWD, int LOGS, int LOG2N, int CL, int RING>
-__global__ void __launch_bounds__(kColThr, (FWD ? SS_COLS_F : SS_COLS_I) * 128 / kColThr) k_ntt16_cols(NttArgs A) {
+__global__ void __launch_bounds__(1 << (LOGS + CL - 4), LOGS + CL == kColTile ? (FWD ? SS_COLS_F : SS_COLS_I) : SS_COLS_BIG)
+    k_ntt16_cols(NttArgs A) {
   enter_grid();
   ntt16_cols<FWD, LOGS, LOG2N, CL, RING>(A, blockIdx.x, blockIdx.y);
 }
@@ -1239,7 +1246,7 @@ __device__ __noinline__ void ntt16_rows_fn(const NttArgs& A, const RowPlan& R, i
 }
 
 template <bool FWD, bool COLS, bool SRC>
-__global__ void __launch_bounds__(COLS ? kColThr : 128, COLS ? 6 * 128 / kColThr : 6) k_ntt16_multi(const __grid_constant__ NttMulti M) {
+__global__ void __launch_bounds__(128, 6) k_ntt16_multi(const __grid_constant__ NttMulti M) {
   for (int t = blockIdx.x; t < M.total; t += gridDim.x) {
     int j = 0;
     while (j + 1 < M.njobs && t >= M.j[j + 1].start) ++j;
@@ -1275,8 +1282,13 @@ __global__ void __launch_bounds__(COLS ? kColThr : 128, COLS ? 6 * 128 / kColThr
 // column phase of one transform by halves
 template <bool FWD, int LOGS, int LOG2N, int RING>
 void launch_cols_as(int npoly, cudaStream_t st, const NttArgs& A) {
-  constexpr int CL = kColTile - LOGS;
-  launch_early(k_ntt16_cols<FWD, LOGS, LOG2N, CL, RING>, dim3(1 << (LOG2N - CL), npoly), kColThr, col_smem<LOGS, CL>(), st, A);
+  constexpr int CL = kColTile - LOGS, CLB = kColTileBig - LOGS;
+  if (((long)npoly << (LOGS + LOG2N - kColTileBig)) >= 2L * SS_COLS_BIG * 152)
+    launch_early(k_ntt16_cols<FWD, LOGS, LOG2N, CLB, RING>, dim3(1 << (LOG2N - CLB), npoly), 256,
+                 col_smem<LOGS, CLB>(), st, A);
+  else
+    launch_early(k_ntt16_cols<FWD, LOGS, LOG2N, CL, RING>, dim3(1 << (LOG2N - CL), npoly), 128, col_smem<LOGS, CL>(), st,
+                 A);
 }
 template <bool FWD>
 void launch_cols(int ring, int logS, int log2n, int npoly, cudaStream_t st, const NttArgs& A) {
@@ -1571,11 +1583,11 @@ void ntt_multi(const std::vector<NttReq>& reqs, bool fwd, cudaStream_t st) {
     Context& C0 = *reqs[b0].C;
     int kr = kt_begin(C0, st);
     if (fwd) {
-      launch_multi<true, true, false>(P1, kColThr, smem_cols, st);
+      launch_multi<true, true, false>(P1, 128, smem_cols, st);
       launch_multi<true, false, false>(P2, thr, smem_rows, st);
     } else {
       launch_multi<false, false, true>(P1, thr, smem_rows, st);
-      launch_multi<false, true, false>(P2, kColThr, smem_cols, st);
+      launch_multi<false, true, false>(P2, 128, smem_cols, st);
     }
     C0.launches += 2;
     if (kr >= 0) C0.kt.ntt_products += prods;
