@@ -831,25 +831,47 @@ __global__ void k_automorph_impl(const u64* a, u64* out, int g, int N, int logN,
 }
 
 // ---------------------------------------------------------------- sampling
+// all 128 output bits mod q; R = 2^64 mod q
+__device__ __forceinline__ u64 uniform_word(u32 index, u32 limb, u32 id, u32 tag, u32 k0, u32 k1, u64 R,
+                                            const Modulus& md) {
+  const Philox4 r = philox(index, limb, id, tag, k0, k1);
+  const u64 lo = ((u64)r.x[1] << 32) | r.x[0];
+  const u64 hi = ((u64)r.x[3] << 32) | r.x[2];
+  // hi 2^64 + lo = (hi mod q) R + lo (mod q), below 2^(2k) + 2^64 <= 2^(63+k) for q of k >= 2 bits
+  Acc128 x{lo, 0};
+  x.mac_wide(barrett_reduce128(0, hi, md), R);
+  return barrett_reduce128(x.hi, x.lo, md);
+}
+
 __global__ void k_uniform_impl(u64* out, long out_os, int nl, int q0, int nq, int L, u32 id0, u32 tag, u32 k0,
-                               u32 k1, int N, const ModDesc* mods) {
+                               u32 k1, int N, const ModDesc* mods, const u64* r64) {
   int poly = blockIdx.y;
   int i = poly % nl, o = poly / nl;
   int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
   int g = i < nq ? q0 + i : L + (i - nq);
   const Modulus& md = MOD(mods, g);
-  Philox4 r = philox((u32)n, (u32)g, id0 + (u32)o, tag, k0, k1);
-  u64 lo = ((u64)r.x[1] << 32) | r.x[0];
-  u64 hi = ((u64)r.x[3] << 32) | r.x[2];
-  // (hi 2^64 + lo) mod q = (hi mod q)(2^64 mod q) + lo mod q
-  u64 R = barrett_reduce128(1, 0, md);
-  u64 h = barrett_reduce128(0, hi, md);
-  u64 v = add_mod(mul_mod(h, R, md), barrett_reduce128(0, lo, md), md.q);
+  const u64 v = uniform_word((u32)n, (u32)g, id0 + (u32)o, tag, k0, k1, __ldg(r64 + kR64 * g), md);
   out[(long)o * out_os + (long)i * N + n] = v;
 }
 
+// Encryption's last step, limb i of ciphertext o: c1 = uniform (the words of
+// k_uniform_impl), c0 = c0 - c1 s. One pass instead of writing c1 and reading it back.
+__global__ void __launch_bounds__(256) k_enc_tail_impl(u64* c0, u64* c1, long os, int L, u32 id0, u32 tag, u32 k0, u32 k1,
+                                                       const u64* s, int N, const ModDesc* mods, const u64* r64) {
+  enter_grid();
+  const int i = blockIdx.y % L, o = blockIdx.y / L;
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= N) return;
+  const Modulus md = MOD(mods, i);
+  const long at = (long)o * os + (long)i * N + n;
+  const u64 a = uniform_word((u32)n, (u32)i, id0 + (u32)o, tag, k0, k1, __ldg(r64 + kR64 * i), md);
+  c1[at] = a;
+  c0[at] = sub_mod(c0[at], mul_mod(a, s[(long)i * N + n], md), md.q);
+}
+
 __global__ void k_cbd_impl(i64* out, u32 id0, u32 tag, u32 k0, u32 k1, int N) {
+  enter_grid();
   int o = blockIdx.y;
   int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
@@ -857,21 +879,31 @@ __global__ void k_cbd_impl(i64* out, u32 id0, u32 tag, u32 k0, u32 k1, int N) {
   out[(long)o * N + n] = (i64)__popc(r.x[0] & 0x1FFFFFu) - (i64)__popc(r.x[1] & 0x1FFFFFu);
 }
 
-// out[o][i] = (m[o] + tmul * e[o]) mod q_g  (coefficient form)
-__global__ void k_lift_small_impl(const i64* e, const u64* m, u64 tmul, u64* out, long out_os, int nl, int q0,
-                                  int nq, int L, int N, const ModDesc* mods) {
-  int poly = blockIdx.y;
-  int i = poly % nl, o = poly / nl;
-  int n = blockIdx.x * blockDim.x + threadIdx.x;
+// out[o][i] = m[o] + tmul * e[o] mod q_g, below 2 q_g (coefficient form), two words a thread
+// for `per` limbs: |e| <= 21 (the sampler's range) and tmul, m < p^r < q / 16 (q = 1
+// mod 2 N p^r, N >= 8), so the value is a signed integer of magnitude below 1.4 q,
+// formed once for all limbs, and lifted by 2q where negative it is below 2q, as the
+// forward transform takes it. (One limb a thread with a modular product read e
+// and m again per limb: 39 us for 8 ciphertexts of 30 limbs of 2^15 words.)
+__global__ void __launch_bounds__(256) k_lift_small_impl(const i64* e, const u64* m, u64 tmul, u64* out, long out_os,
+                                                         int nl, int per, int q0, int nq, int L, int N,
+                                                         const ModDesc* mods) {
+  enter_grid();
+  const int o = blockIdx.y;
+  const int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (n >= N) return;
-  int g = i < nq ? q0 + i : L + (i - nq);
-  const Modulus& md = MOD(mods, g);
-  u64 q = md.q;
-  i64 ev = e ? e[(long)o * N + n] : 0;
-  u64 el = ev >= 0 ? (u64)ev : q - (u64)(-ev);
-  u64 v = mul_mod(el, tmul, md);  // tmul, m < p^r < q (checked at context creation)
-  if (m) v = add_mod(v, m[(long)o * N + n], q);
-  out[(long)o * out_os + (long)i * N + n] = v;
+  i64 v[2];
+#pragma unroll
+  for (int w = 0; w < 2; ++w)
+    v[w] = e[(long)o * N + n + w] * (i64)tmul + (m ? (i64)m[(long)o * N + n + w] : 0);
+  for (int i = blockIdx.z * per; i < min(nl, (int)(blockIdx.z + 1) * per); ++i) {
+    const int g = i < nq ? q0 + i : L + (i - nq);
+    const u64 q = MOD(mods, g).q;
+    u64 r[2];
+#pragma unroll
+    for (int w = 0; w < 2; ++w) r[w] = (u64)v[w] + (v[w] < 0 ? 2 * q : 0);
+    st2(out + (long)o * out_os + (long)i * N + n, r[0], r[1]);
+  }
 }
 
 // out = x - a * s  (evaluation form); s indexed by global prime
@@ -1174,33 +1206,36 @@ __global__ void __launch_bounds__(256) k_lincomb_tiny_impl(const __grid_constant
   enter_grid();
   const int poly = blockIdx.y;  // (bt, comp, i)
   const int i = poly % level, comp = (poly / level) % ncomp, bt = poly / (level * ncomp);
-  const int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  constexpr int V = 2;  // one word a thread: 888 us, two outputs at once: 889 (here 822)
+  const int n = V * (blockIdx.x * blockDim.x + threadIdx.x);
   if (n >= N) return;
   const Modulus md = MOD(mods, i);
   const size_t row = (size_t)(bt * ncomp + comp);
-  u32 yl[2][NT], yh[2][NT];
-  u64 sl[2] = {0, 0}, sh[2] = {0, 0};
+  u32 yl[V][NT], yh[V][NT];
+  u64 sl[V] = {}, sh[V] = {};
 #pragma unroll
   for (int t = 0; t < NT; ++t) {
-    const ulonglong2 y = ld2(A.ptr[t] + (row * A.cap[t] + i) * N + n);
-    yl[0][t] = (u32)y.x & 0x7fffffffu;
-    yh[0][t] = (u32)(y.x >> 31);
-    yl[1][t] = (u32)y.y & 0x7fffffffu;
-    yh[1][t] = (u32)(y.y >> 31);
+    u64 y[V];
+    ldv<V>(A.ptr[t] + (row * A.cap[t] + i) * N + n, y);
 #pragma unroll
-    for (int v = 0; v < 2; ++v) {
+    for (int v = 0; v < V; ++v) {
+      yl[v][t] = (u32)y[v] & 0x7fffffffu;
+      yh[v][t] = (u32)(y[v] >> 31);
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
       sl[v] += yl[v][t];
       sh[v] += yh[v][t];
     }
   }
-  u128 base[2];
+  u128 base[V];
 #pragma unroll
-  for (int v = 0; v < 2; ++v)
+  for (int v = 0; v < V; ++v)
     base[v] = ((u128)md.q << 32) - ((u128)sl[v] << 27) - ((u128)sh[v] << 58);
   for (int j = 0; j < nout; ++j) {
-    u64 r[2];
+    u64 r[V];
 #pragma unroll
-    for (int v = 0; v < 2; ++v) {
+    for (int v = 0; v < V; ++v) {
       u32 l0 = 0, l1 = 0, h0 = 0, h1 = 0;
 #pragma unroll
       for (int t = 0; t < NT; ++t) {
@@ -1210,7 +1245,7 @@ __global__ void __launch_bounds__(256) k_lincomb_tiny_impl(const __grid_constant
       const u128 x = base[v] + (((u64)l1 << 32) | l0) + ((u128)(((u64)h1 << 32) | h0) << 31);
       r[v] = barrett_reduce128((u64)(x >> 64), (u64)x, md);
     }
-    st2(A.out[j] + (row * A.ocap[j] + i) * N + n, r[0], r[1]);
+    stv<V>(A.out[j] + (row * A.ocap[j] + i) * N + n, r);
   }
 }
 
@@ -1602,21 +1637,25 @@ void k_uniform(Context& C, u64* out, long out_os, int n_outer, int nl, int q0, i
   u32 k0, k1;
   seed_words(C, k0, k1);
   k_uniform_impl<<<grid_for(C.N, n_outer * nl), TPB, 0, st>>>(out, out_os, nl, q0, nq, C.L, id0, tag, k0, k1, C.N,
-                                                               C.d_mod);
+                                                               C.d_mod, C.d_r64);
   LAUNCHED();
 }
 
 void k_cbd(Context& C, i64* out, int n_outer, u32 id0, u32 tag, cudaStream_t st) {
   u32 k0, k1;
   seed_words(C, k0, k1);
-  k_cbd_impl<<<grid_for(C.N, n_outer), TPB, 0, st>>>(out, id0, tag, k0, k1, C.N);
+  launch_early(k_cbd_impl, grid_for(C.N, n_outer), TPB, 0, st, out, id0, tag, k0, k1, C.N);
   LAUNCHED();
 }
 
 void k_lift_small(Context& C, const i64* e, const u64* m, u64 tmul, u64* out, long out_os, int n_outer, int nl,
                   int q0, int nq, cudaStream_t st) {
-  k_lift_small_impl<<<grid_for(C.N, n_outer * nl), TPB, 0, st>>>(e, m, tmul, out, out_os, nl, q0, nq, C.L, C.N,
-                                                                  C.d_mod);
+  // all limbs in one thread, or fewer where that leaves SMs without blocks
+  const dim3 b = grid_for(C.N / 2, n_outer);
+  const int parts = (int)std::min((long)nl, std::max(1L, (8L * 152 + b.x * (long)b.y - 1) / (b.x * (long)b.y)));
+  const int per = (nl + parts - 1) / parts;
+  launch_early(k_lift_small_impl, dim3(b.x, b.y, (nl + per - 1) / per), TPB, 0, st, e, m, tmul, out, out_os, nl, per, q0,
+               nq, C.L, C.N, C.d_mod);
   LAUNCHED();
 }
 
@@ -1624,6 +1663,14 @@ void k_mul_sub(Context& C, const u64* x, long x_os, const u64* a, long a_os, con
                int n_outer, int nl, int q0, int nq, int, cudaStream_t st) {
   k_mul_sub_impl<<<grid_for(C.N, n_outer * nl), TPB, 0, st>>>(x, x_os, a, a_os, s, out, out_os, nl, q0, nq, C.L, C.N,
                                                                C.d_mod);
+  LAUNCHED();
+}
+
+void k_enc_tail(Context& C, u64* c0, u64* c1, long os, int n_outer, u32 id0, u32 tag, cudaStream_t st) {
+  u32 k0, k1;
+  seed_words(C, k0, k1);
+  launch_early(k_enc_tail_impl, grid_for(C.N, n_outer * C.L), TPB, 0, st, c0, c1, os, C.L, id0, tag, k0, k1, C.d_sk, C.N,
+               C.d_mod, C.d_r64);
   LAUNCHED();
 }
 

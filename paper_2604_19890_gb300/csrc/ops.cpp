@@ -295,12 +295,11 @@ void op_encrypt(Context& C, const u64* m, int B, u32 nonce0, int t_exp, Buf& out
   const long os = 2L * out.cap * N;
   u64* c0 = out.data;
   u64* c1 = out.data + (size_t)out.cap * N;
-  k_uniform(C, c1, os, B, L, 0, L, nonce0, TAG_ENC_A, st);
   i64* e = static_cast<i64*>(pool_alloc((size_t)B * N * 8, st));
   k_cbd(C, e, B, nonce0, TAG_ENC_E, st);
   k_lift_small(C, e, m, C.tpow[t_exp], c0, os, B, L, 0, L, st);
   ntt_forward(C, PolySet{c0, os, B, L, 0, L}, st);
-  k_mul_sub(C, c0, os, c1, os, C.d_sk, c0, os, B, L, 0, L, 0, st);
+  k_enc_tail(C, c0, c1, os, B, nonce0, TAG_ENC_A, st);
   pool_free(e, st);
 }
 

@@ -327,6 +327,8 @@ void k_lift_small(Context& C, const i64* e, const u64* m, u64 tmul, u64* out, lo
                   int q0, int nq, cudaStream_t st);
 void k_mul_sub(Context& C, const u64* x, long x_os, const u64* a, long a_os, const u64* s, u64* out, long out_os,
                int n_outer, int nl, int q0, int nq, int s_stride_primes, cudaStream_t st);
+// c1 = uniform words, c0 -= c1 s on the data primes ([n_outer] polynomials of stride os)
+void k_enc_tail(Context& C, u64* c0, u64* c1, long os, int n_outer, u32 id0, u32 tag, cudaStream_t st);
 void k_dec_dot(Context& C, const Buf& a, u64* out, cudaStream_t st);
 void k_crt(Context& C, const u64* v, int count, int level, int t_exp, u64* out, cudaStream_t st);
 void k_ksk_gadget(Context& C, u64* b, const u64* sprime, int j, cudaStream_t st);
