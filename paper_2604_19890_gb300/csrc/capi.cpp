@@ -63,6 +63,10 @@ void deliver(ss::Context& C, const ss::BufP& r, ss_ct* out, cudaStream_t st) {
   out->t_exp = r->t_exp;
 }
 
+// The kernels move words in pairs; arrays that start between two 16-byte
+// boundaries go through a pool block where an entry point takes them.
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 ss::Buf as_out(ss_ct* o) {
   ss::Buf b;
   b.data = o->data;
@@ -191,6 +195,12 @@ ss_status ss_encrypt(ss_ctx* ctx, const uint64_t* coeffs, int32_t count, uint32_
   return guard([&] {
     need(ctx && coeffs && out && count >= 1, SS_ERR_PARAM, "bad argument");
     check_out(out, count, 2, ctx->C.L);
+    if (!aligned16(out->data)) {
+      ss::BufP r = ss::alloc_buf(ctx->C, count, 2, ctx->C.L, t_exp, S(stream));
+      ss::op_encrypt(ctx->C, coeffs, count, nonce0, t_exp, *r, S(stream));
+      deliver(ctx->C, r, out, S(stream));
+      return;
+    }
     ss::Buf o = as_out(out);
     ss::op_encrypt(ctx->C, coeffs, count, nonce0, t_exp, o, S(stream));
     write_back(o, out);
@@ -339,6 +349,10 @@ ss_status ss_mul_relin(ss_ctx* ctx, const ss_ct* a, const ss_ct* b, ss_ct* out, 
       ss::ev_mul_into(ctx->C, va, vb, plan, S(stream));
     }
     check_out(out, a->count, 2, std::min(a->level, b->level) - 1);
+    if (!aligned16(out->data)) {
+      deliver(ctx->C, ss::ev_mul(ctx->C, va, vb, S(stream)), out, S(stream));
+      return;
+    }
     ss::Buf o = as_out(out);
     ss::ev_mul_into(ctx->C, va, vb, o, S(stream));
     write_back(o, out);
@@ -569,8 +583,18 @@ static ss_status raw_ntt(ss_ctx* ctx, bool fwd, uint64_t* data, int32_t npoly, i
     need(first >= 0 && first + nprimes <= C.L, SS_ERR_PARAM, "prime range outside the data primes");
     need(npoly % nprimes == 0, SS_ERR_SHAPE, "npoly must be a multiple of nprimes");
     ss::PolySet s{data, (long)nprimes * C.N, npoly / nprimes, nprimes, first, nprimes};
-    if (fwd) ss::ntt_forward(C, s, S(stream));
-    else ss::ntt_inverse(C, s, S(stream));
+    cudaStream_t st = S(stream);
+    const size_t bytes = (size_t)npoly * C.N * 8;
+    if (!aligned16(data)) {
+      s.base = static_cast<uint64_t*>(ss::pool_alloc(bytes, st));
+      SS_CUDA(cudaMemcpyAsync(s.base, data, bytes, cudaMemcpyDeviceToDevice, st));
+    }
+    if (fwd) ss::ntt_forward(C, s, st);
+    else ss::ntt_inverse(C, s, st);
+    if (s.base != data) {
+      SS_CUDA(cudaMemcpyAsync(data, s.base, bytes, cudaMemcpyDeviceToDevice, st));
+      ss::pool_free(s.base, st);
+    }
   });
 }
 

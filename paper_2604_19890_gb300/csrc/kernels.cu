@@ -237,8 +237,9 @@ __device__ __forceinline__ void sum_halves(const u32 (&yl)[NS][V], const u32 (&y
 // dst limb m (global prime g(m) = m < nq ? m : L + m - nq), m outside
 // [skip_lo, skip_hi):  sum_s [src_s * c1_s]_{q_s} * c2[s][g(m)]  (mod q_g), then
 // times post[g] when post != null. Source s lives on prime sp0 + s (s < nsq)
-// or L + s - nsq. Words come out below 3q, as the forward transforms take them
-// (below 4q). NS <= 4 sources, halves of y_s and one Montgomery step by 2^32 as
+// or L + s - nsq. Words come out below 2q (the single-phase transform's folded first
+// stage subtracts them from 2q): sum_s of the halves' products is below NS (2^SPLIT +
+// 2^(bits-SPLIT)) q <= 2^32 q, a Montgomery step by 2^32 leaves below that plus q. NS <= 4 sources, halves of y_s and one Montgomery step by 2^32 as
 // in k_modup; SPLIT low bits keep the low products' sum below 2^64 also for
 // 58-bit primes (8 (2^29 - 1)(2^32 - 1) for NS = 4). Per block, each target's
 // modulus, -q^-1 mod 2^64 and the pairs (c2 post 2^32, c2 post 2^(32+SPLIT)) mod
@@ -415,8 +416,8 @@ __global__ void __launch_bounds__(256) k_bconv_many_impl(const u64* src, long sr
 // l)) converted to the other data primes and the special primes, for every digit
 // in one launch. Output word: sum_s y_s c_s mod q_g, y_s = [x_s c1_s]_{q_s} exact.
 // By halves of y_s (SPLIT low bits l_s, the rest h_s): sum_s l_s c_s0 + h_s c_s1 with
-// c_s0 = c_s 2^32, c_s1 = c_s 2^(32+SPLIT) mod q_g, below (NS / 4 + ..) 2^32 q_g, and one
-// Montgomery step by 2^32; the result is below 3 q_g, as the forward transform that
+// c_s0 = c_s 2^32, c_s1 = c_s 2^(32+SPLIT) mod q_g, below (NS / 4 + ..) 2^32 q_g < 2^32 q_g, and one
+// Montgomery step by 2^32; the result is below 2 q_g, as the forward transform that
 // reads it takes. SPLIT leaves the low products' sum below 2^64, so a target costs
 // 4 NS + 2 accumulating 64-bit products and one 32-bit one (58 cycles of the multiply
 // pipe a warp for NS = 3) where 128-bit sums and a Montgomery step by 2^64 took 72 and

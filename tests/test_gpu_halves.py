@@ -120,3 +120,40 @@ def test_small_coefficient_combinations(bits, logN, nin, nout):
             q = int(g.primes[i])
             exp = sum(int(rows[j, t]) * w[t, 0, :, i, :].astype(object) for t in range(nin)) % q
             assert (got[:, i, :].astype(object) == exp).all(), (j, i)
+
+
+@pytest.mark.parametrize("logN", [9, 13])
+def test_arrays_between_16_byte_boundaries(logN):
+    """The raw transform, the encryption and the multiplication take outputs that start on any word."""
+    import ctypes as C
+
+    import torch
+
+    import paper_2604_19890_gb300 as ssg
+    g = ssg.Context(logN=logN, L=3, alpha=2, bits=50, p=17, r=1, h=8, seed=31, nmax=0)
+    g.keygen([])
+    rng = np.random.default_rng(logN)
+    data = np.stack([rng.integers(0, int(g.primes[i % 3]), g.N, dtype=np.uint64) for i in range(6)])
+    even = torch.from_numpy(data.view(np.int64).copy()).cuda()
+    odd = torch.zeros(6 * g.N + 1, dtype=torch.int64, device="cuda")[1:]
+    odd.copy_(even.flatten())
+    assert odd.data_ptr() % 16 == 8
+    for f in (g.ntt_forward, g.ntt_inverse):
+        f(even, 0, 3)
+        f(odd, 0, 3)
+        assert torch.equal(odd, even.flatten())
+    m = np.stack([g.encode(rng.integers(0, g.t, g.slots)) for _ in range(2)])
+    a = g.encrypt(m, 5)
+    flat = torch.zeros(a.buf.numel() + 1, dtype=torch.int64, device="cuda")[1:]
+    d = a.desc()
+    d.data = flat.data_ptr()
+    dm = torch.from_numpy(m.view(np.int64).copy()).cuda()
+    st = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert ssg.lib().ss_encrypt(g.h, C.c_void_p(dm.data_ptr()), 2, 5, a.t_exp, C.byref(d), st) == ssg.SS_OK
+    assert torch.equal(flat, a.buf.flatten())
+    p = g.mul_relin(a, a)
+    flat = torch.zeros(p.buf.numel() + 1, dtype=torch.int64, device="cuda")[1:]
+    da, do = a.desc(), p.desc()
+    do.data = flat.data_ptr()
+    assert ssg.lib().ss_mul_relin(g.h, C.byref(da), C.byref(da), C.byref(do), st) == ssg.SS_OK
+    assert torch.equal(flat, p.buf.flatten()) and (do.level, do.ncomp) == (p.level, p.ncomp)
