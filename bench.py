@@ -30,18 +30,18 @@ FALLBACK_HBM = 6800.0
 # 16-lane fmaheavy pipe = 64 multiply issue slots per SM per clock, at the
 # 2070 MHz maximum SM clock.
 IMAD_PEAK = 152 * 64 * 2.07e9
-# 32-bit multiplies in one 64-bit Shoup butterfly product (schoolbook minimum):
-# the high 64 bits of a*w' need the high half of aL*wL and the full products
-# aL*wH, aH*wL, aH*wH; the low 64 bits of a*w and of qhat*q each need one full
-# product and two low halves. 5 of the 10 are widening (32 x 32 -> 64) products;
-# their cost in issue slots is the measured ratio of the 32-bit and widening
-# multiply-add rates (probe kinds 0 and 2).
-IMAD_PER_BUTTERFLY = 10
+# 32-bit multiplies in one butterfly product of the transforms (products by halves:
+# a = h 2^32 + l against w and 2^32 w mod q): the 32-bit quotient takes two
+# widening (32 x 32 -> 64) products, the low 64 bits of l w, h (2^32 w) and of the
+# quotient times 2q one widening product and one low half each. 5 of the 8 are
+# widening; their cost in issue slots is the measured ratio of the 32-bit and
+# widening multiply-add rates (probe kinds 0 and 2).
+IMAD_PER_BUTTERFLY = 8
 WIDE_PER_BUTTERFLY = 5
-# DRAM bytes per limb transform (forward and inverse, both phases each) from one
-# ncu capture of the transform kernels (dram__bytes_read.sum +
-# dram__bytes_write.sum per limb), over the 1 MB (16 N) it must move.
-NTT_TRAFFIC_PER_ALGO_BYTE = 1.860
+# DRAM bytes that the transform launches and the fused inner product move per
+# algorithmic byte of the two classes, from one ncu capture of a multiplication of
+# four ciphertexts at N = 2^16, level 41 (dram__bytes_read.sum + dram__bytes_write.sum).
+NTT_TRAFFIC_PER_ALGO_BYTE = 1.021
 
 
 def hbm_peak():
@@ -724,18 +724,22 @@ def run_ours(args):
         return b / (ms / 1e3) / 1e9 if ms > 0 else 0.0
 
     n_l, ms_l, b_l = ks[dom]
-    if dom == "ntt":
-        # integer-multiply roofline of the transform: the Shoup products its
+    # the chunk phase of a key switch's digits runs inside the inner-product launches
+    # (one kernel): the transforms' roofline takes both classes together
+    both = {"ntt", "keyswitch_inner_product"}
+    if dom in both:
+        n_l, ms_l, b_l = (sum(ks[k][i] for k in both) for i in range(3))
+        # integer-multiply roofline of the transforms: the butterfly products their
         # launches performed (N/2 per stage and limb; fewer where the ModUp base
         # conversion applied the first twiddle), counted by the library
         bfly = ntt_products
         achieved = bfly * slots_per_bfly / (ms_l / 1e3) / 1e12
         peak_alu = IMAD_PEAK / 1e12
-        roof = {"kernel": "ntt", "bound": "alu", "achieved": achieved, "peak": peak_alu,
+        roof = {"kernel": "ntt + fused inner product", "bound": "alu", "achieved": achieved, "peak": peak_alu,
                 "unit": "T multiply issue slots/s", "frac": achieved / peak_alu,
                 "traffic": (NTT_TRAFFIC_PER_ALGO_BYTE * b_l / n_l) if NTT_TRAFFIC_PER_ALGO_BYTE else None,
-                "peak_source": "derived: 152 SMs x 64 multiply issue slots/clk x 2070 MHz; per Shoup product "
-                               "10 multiplies = 5 single-slot + 5 widening at the measured slot ratio "
+                "peak_source": "derived: 152 SMs x 64 multiply issue slots/clk x 2070 MHz; per product "
+                               "8 multiplies = 3 single-slot + 5 widening at the measured slot ratio "
                                "(%.2f slots each), %.2f slots" % (wide_slots, slots_per_bfly),
                 "shoup_products": bfly,
                 "frac_at_one_slot_per_multiply": bfly * IMAD_PER_BUTTERFLY / (ms_l / 1e3) / IMAD_PEAK,
@@ -743,7 +747,8 @@ def run_ours(args):
                 "measured_butterflies_per_s": bfly_rate,
                 "achieved_butterflies_per_s": bfly / (ms_l / 1e3),
                 "frac_of_measured_butterfly_ceiling": bfly / (ms_l / 1e3) / bfly_rate,
-                "hbm_achieved_gbs": gbs(dom), "hbm_peak_gbs": peak, "hbm_frac": gbs(dom) / peak,
+                "hbm_achieved_gbs": b_l / (ms_l / 1e3) / 1e9, "hbm_peak_gbs": peak,
+                "hbm_frac": b_l / (ms_l / 1e3) / 1e9 / peak,
                 "hbm_peak_source": peak_kind, "avg_launch_ms": ms_l / max(1, n_l),
                 "algorithmic_bytes_per_launch": b_l / max(1, n_l),
                 "share_of_kernel_time": ms_l / total_k if total_k else None}

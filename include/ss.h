@@ -360,8 +360,10 @@ int32_t ss_trace_get(ss_ctx* ctx, char* buf, int32_t len);
  * When on, every library kernel launch is bracketed by CUDA events recorded on
  * the stream it is launched on, and attributed to a class with the bytes the
  * operation must move (its algorithmic traffic, not the measured traffic):
- *   0 NTT (both phases of one transform; 16 N bytes per limb)
- *   1 base conversion   2 key-switch inner product   3 tensor product
+ *   0 NTT (both phases of one transform, or the column phase of a key switch's
+ *     digits and correction; 16 N bytes per limb)
+ *   1 base conversion   2 key-switch inner product (N >= 8192, primes below
+ *     2^55: fused with the chunk phase of those transforms)   3 tensor product
  *   4 subtract-and-scale (ModDown / modulus-switch epilogue)
  *   5 automorphism   6 other elementwise   7 sampling.
  * ss_kernel_stats synchronises on the recorded events and returns, for one
@@ -370,9 +372,9 @@ int32_t ss_trace_get(ss_ctx* ctx, char* buf, int32_t len);
 ss_status ss_kernel_timing(ss_ctx* ctx, int32_t on);
 ss_status ss_kernel_stats(ss_ctx* ctx, int32_t cls, uint64_t* launches, double* ms, double* bytes);
 
-/* Shoup products (one 64-bit modular product by a precomputed constant each)
- * that the timed transform launches performed since kernel timing was switched
- * on: per polynomial N/2 log2 N forward, less N/2 when the base conversion
+/* Products (one 64-bit modular product by a precomputed constant each) that the
+ * timed transforms performed, those finished inside the fused inner product
+ * included, since kernel timing was switched on: per polynomial N/2 log2 N forward, less N/2 when the base conversion
  * that wrote the input already applied the first stage's twiddle (ring
  * X^N + 1), and N/2 (log2 N + 1) inverse for N > 4096 (the last stage also
  * scales the sums by N^-1), N/2 (log2 N + 2) for N <= 4096 (N^-1 on every
