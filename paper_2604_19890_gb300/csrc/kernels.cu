@@ -239,8 +239,8 @@ __device__ __forceinline__ void sum_halves(const u32 (&yl)[NS][V], const u32 (&y
 // times post[g] when post != null. Source s lives on prime sp0 + s (s < nsq)
 // or L + s - nsq. Words come out below 2q (the single-phase transform's folded first
 // stage subtracts them from 2q): sum_s of the halves' products is below NS (2^SPLIT +
-// 2^(bits-SPLIT)) q <= 2^32 q, a Montgomery step by 2^32 leaves below that plus q. NS <= 4 sources, halves of y_s and one Montgomery step by 2^32 as
-// in k_modup; SPLIT low bits keep the low products' sum below 2^64 also for
+// 2^(bits-SPLIT)) q <= 2^32 q, a Montgomery step by 2^32 leaves below that plus q. NS <= 4
+// sources, halves of y_s and one Montgomery step by 2^32 as in k_modup; SPLIT low bits keep the low products' sum below 2^64 also for
 // 58-bit primes (8 (2^29 - 1)(2^32 - 1) for NS = 4). Per block, each target's
 // modulus, -q^-1 mod 2^64 and the pairs (c2 post 2^32, c2 post 2^(32+SPLIT)) mod
 // q_g are staged once in shared memory (row m: q, -q^-1, the pairs), one thread a
@@ -1126,7 +1126,8 @@ struct LinMultiArgs {
 };
 
 // Two consecutive words per thread.
-__global__ void __launch_bounds__(256) k_lincomb_multi_impl(LinMultiArgs A, int nin, int nout, int small, int N, int ncomp, int level, const ModDesc* mods) {
+__global__ void __launch_bounds__(256) k_lincomb_multi_impl(LinMultiArgs A, int nin, int nout, int small, int N,
+                                                            int ncomp, int level, const ModDesc* mods) {
   enter_grid();
   const int poly = blockIdx.y;  // (bt, comp, i)
   const int i = poly % level, comp = (poly / level) % ncomp, bt = poly / (level * ncomp);
@@ -1310,7 +1311,8 @@ void k_lincomb(Context& C, const std::vector<const Buf*>& ys, const std::vector<
   }
   int polys = out.count * out.ncomp * out.level;
   TIMED(KC_ELEM, (nt + 1.0) * polys * C.N * 8.0,
-        launch_early(k_lincomb_impl, grid_for(C.N / 2, polys), TPB, 0, st, A, nt, cst, small ? npos + 1 : 0, tiny ? 1 : 0, out.data,
+        launch_early(k_lincomb_impl, grid_for(C.N / 2, polys), TPB, 0, st,
+                     A, nt, cst, small ? npos + 1 : 0, tiny ? 1 : 0, out.data,
                                                                   out.cap, C.N,
                                                               out.ncomp, out.level, C.d_mod));
   LAUNCHED();
@@ -1346,7 +1348,8 @@ void k_lincomb_multi(Context& C, const std::vector<const Buf*>& ys, const std::v
   const double bytes = (double)(nin + nout) * polys * C.N * 8.0;
   if (!tiny) {
     TIMED(KC_ELEM, bytes,
-          launch_early(k_lincomb_multi_impl, grid_for(C.N / 2, polys), TPB, 0, st, A, nin, nout, small ? 1 : 0, C.N, o0.ncomp,
+          launch_early(k_lincomb_multi_impl, grid_for(C.N / 2, polys), TPB, 0, st,
+                       A, nin, nout, small ? 1 : 0, C.N, o0.ncomp,
                                                                         o0.level, C.d_mod));
     LAUNCHED();
     return;
@@ -1383,7 +1386,8 @@ void k_batch_sum(Context& C, const Buf& a, Buf& out, cudaStream_t st) {
 void k_binary(Context& C, int op, const Buf& a, const Buf& b, Buf& out, cudaStream_t st) {
   int polys = a.count * a.ncomp * a.level;
   TIMED(KC_ELEM, 3.0 * polys * (double)C.N * 8.0,
-  launch_early(k_binary_impl, grid_for(C.N / 2, polys), TPB, 0, st, op, a.data, b.data, out.data, C.N, a.ncomp, a.level, a.cap,
+  launch_early(k_binary_impl, grid_for(C.N / 2, polys), TPB, 0, st,
+               op, a.data, b.data, out.data, C.N, a.ncomp, a.level, a.cap,
                                                        b.cap, out.cap, b.count == 1 && a.count > 1, C.d_mod));
   LAUNCHED();
 }
@@ -1406,7 +1410,8 @@ void k_copy_limbs(Context& C, const Buf& a, Buf& out, int level, cudaStream_t st
 void k_tensor(Context& C, const Buf& a, const Buf& b, Buf& out, cudaStream_t st) {
   int polys = a.count * a.level;
   TIMED(KC_TENSOR, 7.0 * polys * (double)C.N * 8.0,
-  launch_early(k_tensor_impl, grid_for(C.N / 2, polys), TPB, 0, st, a.data, b.data, out.data, C.N, a.level, a.cap, b.cap, out.cap,
+  launch_early(k_tensor_impl, grid_for(C.N / 2, polys), TPB, 0, st,
+               a.data, b.data, out.data, C.N, a.level, a.cap, b.cap, out.cap,
                                                        C.d_mod));
   LAUNCHED();
 }
@@ -1432,7 +1437,7 @@ void k_bconv(Context& C, const u64* src, long src_os, int ns, int sp0, const u64
   switch (ns) {
     SS_BCONV(1) SS_BCONV(2) SS_BCONV(3) SS_BCONV(4)
     default:
-      launch_early(k_bconv_many_impl<4, 2>, dim3((g.x + 1) / 2, g.y), TPB, smem, st, 
+      launch_early(k_bconv_many_impl<4, 2>, dim3((g.x + 1) / 2, g.y), TPB, smem, st,
           src, src_os, ns, sp0, nsq, c1, c2, C.ntot, dst, dst_os, nd, nq, C.L, skip_lo, skip_hi, post, C.N, C.d_mod,
           C.d_r64, pre, dscale);
       break;
@@ -1466,7 +1471,8 @@ void k_modup(Context& C, const u64* src, u64* dst, int level, int B, cudaStream_
 void k_sub_scale(Context& C, const u64* a, long a_os, const u64* dl, long d_os, const u64* scale, const u64* add,
                  long add_os, u64* out, long out_os, int nl, int n_outer, cudaStream_t st) {
   TIMED(KC_SUBSCALE, (add ? 4.0 : 3.0) * nl * n_outer * (double)C.N * 8.0,
-  launch_early(k_sub_scale_impl, grid_for(C.N / 2, nl * n_outer), TPB, 0, st, a, a_os, dl, d_os, scale, add, add_os, out, out_os,
+  launch_early(k_sub_scale_impl, grid_for(C.N / 2, nl * n_outer), TPB, 0, st,
+               a, a_os, dl, d_os, scale, add, add_os, out, out_os,
                                                                  nl, C.N, C.d_mod));
   LAUNCHED();
 }
@@ -1619,11 +1625,11 @@ void ks_multi(const std::vector<KsReq>& reqs, cudaStream_t st) {
 void k_automorph(Context& C, const Buf& a, int g, Buf& out, cudaStream_t st) {
   int rows = a.count * a.ncomp;
   TIMED(KC_AUTOMORPH, 2.0 * rows * a.level * (double)C.N * 8.0,
-  if (C.m_odd == 5) launch_early(k_automorph_impl<5>, grid_for(C.N, rows * a.level), TPB, 0, st, 
+  if (C.m_odd == 5) launch_early(k_automorph_impl<5>, grid_for(C.N, rows * a.level), TPB, 0, st,
       a.data, out.data, g, C.N, C.logN, rows, a.cap, out.cap, a.level);
-  else if (C.m_odd == 3) launch_early(k_automorph_impl<3>, grid_for(C.N, rows * a.level), TPB, 0, st, 
+  else if (C.m_odd == 3) launch_early(k_automorph_impl<3>, grid_for(C.N, rows * a.level), TPB, 0, st,
       a.data, out.data, g, C.N, C.logN, rows, a.cap, out.cap, a.level);
-  else launch_early(k_automorph_impl<1>, grid_for(C.N, rows * a.level), TPB, 0, st, 
+  else launch_early(k_automorph_impl<1>, grid_for(C.N, rows * a.level), TPB, 0, st,
       a.data, out.data, g, C.N, C.logN, rows, a.cap, out.cap, a.level));
   LAUNCHED();
 }

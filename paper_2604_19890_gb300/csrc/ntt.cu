@@ -797,51 +797,51 @@ __device__ __forceinline__ void ntt16_cols(const NttArgs& A, int tile, int poly)
     for (int k = 0; k < 16; ++k) col[(16 * rest + (long)k) * STRIDE] = x[k];
   } else {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) half_stage<false>(x, j, j, twS, tpS, hm, false, narrow_slot);
-  half_settle(x, 4, hm);
+    for (int j = 0; j < 4; ++j) half_stage<false>(x, j, j, twS, tpS, hm, false, narrow_slot);
+    half_settle(x, 4, hm);
 #pragma unroll
-  for (int k = 0; k < 16; ++k) data[col_swz<CL>(((16 * rest + k) << CL) + c)] = x[k];
-  __syncthreads();
+    for (int k = 0; k < 16; ++k) data[col_swz<CL>(((16 * rest + k) << CL) + c)] = x[k];
+    __syncthreads();
 #pragma unroll
-  for (int k = 0; k < 16; ++k) x[k] = data[col_swz<CL>(((rest + G * k) << CL) + c)];
-  constexpr int NS = LOGS - 4;  // stages j = 4 - NS .. 3, the last one (or two) with N^-1
-  constexpr int JE = RING == 5 ? 2 : 3;
-  if constexpr (4 - NS < JE) {
+    for (int k = 0; k < 16; ++k) x[k] = data[col_swz<CL>(((rest + G * k) << CL) + c)];
+    constexpr int NS = LOGS - 4;  // stages j = 4 - NS .. 3, the last one (or two) with N^-1
+    constexpr int JE = RING == 5 ? 2 : 3;
+    if constexpr (4 - NS < JE) {
 #pragma unroll
-    for (int j = 4 - NS; j < JE; ++j) half_stage<false>(x, j, j - (4 - NS), twS, tpS, hm, false, wide_slot);
-  }
-  const u64* nv = A.ninv + 6 * pidx;
-  const u64 off = q << (5 + NS - 1);  // above every input of the last stage
-  if (RING == 5) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) split4_inv(x[k], x[k + 4], x[k + 8], x[k + 12], spl, q, off);
-  } else if (RING == 3) {
-    const u64 ni = nv[0], nip = nv[1], w = nv[2], wp = nv[3], cn = nv[4], cnp = nv[5];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const u64 sv = x[k] + x[k + 8], dv = x[k] - x[k + 8] + off;
-      const u64 lo = shoup(sv, ni, nip, q), cr = shoup(dv, cn, cnp, q);
-      x[k] = lo >= cr ? lo - cr : lo + q - cr;
-      x[k + 8] = shoup(dv, w, wp, q);
+      for (int j = 4 - NS; j < JE; ++j) half_stage<false>(x, j, j - (4 - NS), twS, tpS, hm, false, wide_slot);
     }
-  } else if (A.post_scale) {  // N^-1 and N^-1 psi^(-N/2) left to the consumer
+    const u64* nv = A.ninv + 6 * pidx;
+    const u64 off = q << (5 + NS - 1);  // above every input of the last stage
+    if (RING == 5) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const u64 U = x[k], V = x[k + 8];
-      x[k] = U + V;
-      x[k + 8] = U - V + off;
+      for (int k = 0; k < 4; ++k) split4_inv(x[k], x[k + 4], x[k + 8], x[k + 12], spl, q, off);
+    } else if (RING == 3) {
+      const u64 ni = nv[0], nip = nv[1], w = nv[2], wp = nv[3], cn = nv[4], cnp = nv[5];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const u64 sv = x[k] + x[k + 8], dv = x[k] - x[k + 8] + off;
+        const u64 lo = shoup(sv, ni, nip, q), cr = shoup(dv, cn, cnp, q);
+        x[k] = lo >= cr ? lo - cr : lo + q - cr;
+        x[k + 8] = shoup(dv, w, wp, q);
+      }
+    } else if (A.post_scale) {  // N^-1 and N^-1 psi^(-N/2) left to the consumer
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const u64 U = x[k], V = x[k + 8];
+        x[k] = U + V;
+        x[k + 8] = U - V + off;
+      }
+    } else {
+      const u64 ni = nv[0], nip = nv[1], w = nv[2], wp = nv[3];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const u64 U = x[k], V = x[k + 8];
+        x[k] = shoup(U + V, ni, nip, q);
+        x[k + 8] = shoup(U - V + off, w, wp, q);
+      }
     }
-  } else {
-    const u64 ni = nv[0], nip = nv[1], w = nv[2], wp = nv[3];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const u64 U = x[k], V = x[k + 8];
-      x[k] = shoup(U + V, ni, nip, q);
-      x[k + 8] = shoup(U - V + off, w, wp, q);
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < 16; ++k) col[(rest + (long)G * k) * STRIDE] = x[k];
+    for (int k = 0; k < 16; ++k) col[(rest + (long)G * k) * STRIDE] = x[k];
   }
 }
 
@@ -1658,7 +1658,8 @@ void rows_ip(Context& C, const RowsIpReq& R, cudaStream_t st) {
   int thr = (A.nb * rpc * tpr + 31) / 32 * 32;
   if ((long)g.x * g.y <= SS_ROWS_IP * 152L) thr = 256;
   const size_t smem = ((size_t)24 << l2) + (size_t)(thr / tpr) * 8 * (1 << l2);
-  const double words = (double)A.dn * R.nlimbs * (R.B + 2.0) + (R.type == 0 ? 2.0 : 4.0 + (R.x ? 2.0 : 0.0)) * R.nlimbs * R.B;
+  const double words = (double)A.dn * R.nlimbs * (R.B + 2.0) +
+                       (R.type == 0 ? 2.0 : 4.0 + (R.x ? 2.0 : 0.0)) * R.nlimbs * R.B;
   int kr = kt_begin(C, st);
   if (l2 == 7) {
     if (R.type == 0) launch_early(k_rows_ip<7, 0>, g, thr, smem, st, A);
