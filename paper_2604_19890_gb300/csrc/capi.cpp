@@ -584,17 +584,15 @@ static ss_status raw_ntt(ss_ctx* ctx, bool fwd, uint64_t* data, int32_t npoly, i
     need(npoly % nprimes == 0, SS_ERR_SHAPE, "npoly must be a multiple of nprimes");
     ss::PolySet s{data, (long)nprimes * C.N, npoly / nprimes, nprimes, first, nprimes};
     cudaStream_t st = S(stream);
-    const size_t bytes = (size_t)npoly * C.N * 8;
-    if (!aligned16(data)) {
-      s.base = static_cast<uint64_t*>(ss::pool_alloc(bytes, st));
-      SS_CUDA(cudaMemcpyAsync(s.base, data, bytes, cudaMemcpyDeviceToDevice, st));
+    const size_t words = aligned16(data) ? 0 : (size_t)npoly * C.N;
+    const ss::PoolWords block(words, st);
+    if (words) {
+      s.base = block.p;
+      SS_CUDA(cudaMemcpyAsync(s.base, data, words * 8, cudaMemcpyDeviceToDevice, st));
     }
     if (fwd) ss::ntt_forward(C, s, st);
     else ss::ntt_inverse(C, s, st);
-    if (s.base != data) {
-      SS_CUDA(cudaMemcpyAsync(data, s.base, bytes, cudaMemcpyDeviceToDevice, st));
-      ss::pool_free(s.base, st);
-    }
+    if (words) SS_CUDA(cudaMemcpyAsync(data, s.base, words * 8, cudaMemcpyDeviceToDevice, st));
   });
 }
 

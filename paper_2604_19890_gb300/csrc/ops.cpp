@@ -92,14 +92,14 @@ static PolySet scaled_later(PolySet s, bool post) {
 // of four of each): the digits, the sums of the dropped limbs, and a region that
 // holds the digit source up to the ModUp and the correction afterwards.
 struct KsScratch {
+  PoolWords block;
   u64 *ext, *acc, *dc, *delta;
-  cudaStream_t st;
-  KsScratch(size_t ext_words, size_t acc_words, size_t dc_words, size_t delta_words, cudaStream_t s) : st(s) {
-    ext = static_cast<u64*>(pool_alloc((ext_words + acc_words + std::max(dc_words, delta_words)) * 8, s));
+  KsScratch(size_t ext_words, size_t acc_words, size_t dc_words, size_t delta_words, cudaStream_t s)
+      : block(ext_words + acc_words + std::max(dc_words, delta_words), s) {
+    ext = block.p;
     acc = ext + ext_words;
     dc = delta = acc + acc_words;
   }
-  ~KsScratch() { pool_free(ext, st); }
 };
 
 // ModUp of every digit: one launch where the context has its table (N >= 8192,
@@ -252,7 +252,8 @@ void op_modswitch(Context& C, const Buf& a, int k, Buf& out, cudaStream_t st) {
   out.ncomp = nc;
   out.level = nl;
   out.t_exp = a.t_exp;
-  u64* x = static_cast<u64*>(pool_alloc((size_t)B * nc * (k + nl) * N * 8, st));
+  const PoolWords scratch((size_t)B * nc * (k + nl) * N, st);
+  u64* x = scratch.p;
   u64* delta = x + (size_t)B * nc * k * N;
   const bool pre = bconv_folds_w1(C), post = bconv_folds_inverse(C);
   ntt_inverse_from(C, scaled_later(PolySet{x, (long)k * N, B * nc, k, nl, k}, post), a.data + (size_t)nl * N,
@@ -268,7 +269,6 @@ void op_modswitch(Context& C, const Buf& a, int k, Buf& out, cudaStream_t st) {
   ntt_forward(C, pd, st);
   k_sub_scale(C, a.data, (long)a.cap * N, delta, (long)nl * N, qinv, nullptr, 0, out.data, (long)out.cap * N, nl,
               B * nc, st);
-  pool_free(x, st);
 }
 
 void op_rotate(Context& C, const Buf& a, int g, Buf& out, cudaStream_t st) {
@@ -295,23 +295,23 @@ void op_encrypt(Context& C, const u64* m, int B, u32 nonce0, int t_exp, Buf& out
   const long os = 2L * out.cap * N;
   u64* c0 = out.data;
   u64* c1 = out.data + (size_t)out.cap * N;
-  i64* e = static_cast<i64*>(pool_alloc((size_t)B * N * 8, st));
+  const PoolWords scratch((size_t)B * N, st);
+  i64* e = reinterpret_cast<i64*>(scratch.p);
   k_cbd(C, e, B, nonce0, TAG_ENC_E, st);
   k_lift_small(C, e, m, C.tpow[t_exp], c0, os, B, L, 0, L, st);
   ntt_forward(C, PolySet{c0, os, B, L, 0, L}, st);
   k_enc_tail(C, c0, c1, os, B, nonce0, TAG_ENC_A, st);
-  pool_free(e, st);
 }
 
 void op_decrypt(Context& C, const Buf& a, u64* d_out, cudaStream_t st) {
   if (!C.have_keys) throw Error(SS_ERR_PARAM, "no keys");
   const int N = C.N, l = a.level, B = a.count;
-  u64* v = static_cast<u64*>(pool_alloc((size_t)B * l * N * 8, st));
+  const PoolWords scratch((size_t)B * l * N, st);
+  u64* v = scratch.p;
   k_dec_dot(C, a, v, st);
   ntt_inverse(C, PolySet{v, (long)l * N, B, l, 0, l}, st);
   SS_CUDA(cudaMemsetAsync(d_out, 0, (size_t)B * N * 8, st));
   k_crt(C, v, B, l, a.t_exp, d_out, st);
-  pool_free(v, st);
 }
 
 // ------------------------------------------------------------------ keys
@@ -336,7 +336,8 @@ static void make_ksk(Context& C, const u64* sprime, u32 key_id, KeyDev& K, cudaS
   size_t words = (size_t)dn * T * N;
   SS_CUDA(cudaMalloc(&K.a, words * 8));
   SS_CUDA(cudaMalloc(&K.b, words * 8));
-  i64* e = static_cast<i64*>(pool_alloc((size_t)N * 8, st));
+  const PoolWords scratch(N, st);
+  i64* e = reinterpret_cast<i64*>(scratch.p);
   for (int j = 0; j < dn; ++j) {
     u32 id = key_id * 256u + (u32)j;
     u64* a = K.a + (size_t)j * T * N;
@@ -350,7 +351,6 @@ static void make_ksk(Context& C, const u64* sprime, u32 key_id, KeyDev& K, cudaS
   }
   k_to_montgomery(C, K.a, dn * T, st);
   k_to_montgomery(C, K.b, dn * T, st);
-  pool_free(e, st);
 }
 
 void op_keygen(Context& C, const std::vector<int>& galois) {
@@ -384,12 +384,11 @@ void op_keygen(Context& C, const std::vector<int>& galois) {
   sview.cap = T;
   for (int g : galois) {
     if (C.gk.count(g)) continue;
-    u64* sg = static_cast<u64*>(pool_alloc((size_t)T * N * 8, st));
+    const PoolWords sg((size_t)T * N, st);
     Buf o = sview;
-    o.data = sg;
+    o.data = sg.p;
     k_automorph(C, sview, g, o, st);
-    make_ksk(C, sg, (u32)g, C.gk[g], st);
-    pool_free(sg, st);
+    make_ksk(C, sg.p, (u32)g, C.gk[g], st);
   }
   SS_CUDA(cudaStreamSynchronize(st));
   C.have_keys = true;

@@ -200,6 +200,15 @@ BufP view_buf(const ss_ct& c);
 BufP slice_buf(const BufP& a, int b0, int count, int N);
 void* pool_alloc(size_t bytes, cudaStream_t s);
 void pool_free(void* p, cudaStream_t s);
+// Pool words held by a scope, given back on every way out of it (a later step may throw).
+struct PoolWords {
+  u64* p;
+  cudaStream_t st;
+  PoolWords(size_t words, cudaStream_t s) : p(static_cast<u64*>(pool_alloc(words * 8, s))), st(s) {}
+  ~PoolWords() { pool_free(p, st); }
+  PoolWords(const PoolWords&) = delete;
+  PoolWords& operator=(const PoolWords&) = delete;
+};
 
 // ------------------------------------------------------------------ launchers
 // Whether the calling thread launches without overlapping a kernel's start with
