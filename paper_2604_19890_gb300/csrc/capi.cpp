@@ -63,8 +63,8 @@ void deliver(ss::Context& C, const ss::BufP& r, ss_ct* out, cudaStream_t st) {
   out->t_exp = r->t_exp;
 }
 
-// The kernels move words in pairs; arrays that start between two 16-byte
-// boundaries go through a pool block where an entry point takes them.
+// Kernels that move words in pairs need 16-byte boundaries; arrays that start
+// between two go through a pool block where an entry point takes them.
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 ss::Buf as_out(ss_ct* o) {
@@ -584,7 +584,8 @@ static ss_status raw_ntt(ss_ctx* ctx, bool fwd, uint64_t* data, int32_t npoly, i
     need(npoly % nprimes == 0, SS_ERR_SHAPE, "npoly must be a multiple of nprimes");
     ss::PolySet s{data, (long)nprimes * C.N, npoly / nprimes, nprimes, first, nprimes};
     cudaStream_t st = S(stream);
-    const size_t words = aligned16(data) ? 0 : (size_t)npoly * C.N;
+    // only the chunk phase of products by halves moves pairs; the other forms work in place on any word
+    const size_t words = aligned16(data) || !C.d_tp ? 0 : (size_t)npoly * C.N;
     const ss::PoolWords block(words, st);
     if (words) {
       s.base = block.p;

@@ -1,5 +1,5 @@
 """Device scratch of single calls: a call that is refused gives back what it took from the
-stream-ordered pool."""
+stream-ordered pool, and a transform in place takes nothing where its kernels read single words."""
 import ctypes as C
 
 import numpy as np
@@ -7,7 +7,7 @@ import pytest
 
 pytestmark = pytest.mark.gpu
 
-USED_CURRENT = 7  # CU_MEMPOOL_ATTR_USED_MEM_CURRENT
+USED_CURRENT, USED_HIGH = 7, 8  # CU_MEMPOOL_ATTR_USED_MEM_CURRENT, CU_MEMPOOL_ATTR_USED_MEM_HIGH
 
 
 class Pool:
@@ -22,11 +22,15 @@ class Pool:
         assert self.cu.cuDeviceGet(C.byref(dev), torch.cuda.current_device()) == 0
         assert self.cu.cuDeviceGetDefaultMemPool(C.byref(self.pool), dev) == 0
 
-    def get(self):
+    def get(self, attr=USED_CURRENT):
         self.torch.cuda.synchronize()
         v = C.c_uint64()
-        assert self.cu.cuMemPoolGetAttribute(self.pool, USED_CURRENT, C.byref(v)) == 0
+        assert self.cu.cuMemPoolGetAttribute(self.pool, attr, C.byref(v)) == 0
         return v.value
+
+    def reset_high(self):
+        v = C.c_uint64(0)
+        assert self.cu.cuMemPoolSetAttribute(self.pool, USED_HIGH, C.byref(v)) == 0
 
 
 def context(**kw):
@@ -63,3 +67,22 @@ def test_refused_raw_transform_gives_back_its_scratch():
         with pytest.raises(ssg.SSError):
             f(odd, 0, 1)
         assert pool.get() == before
+
+
+# single-phase transforms and the form of wide primes read words one by one, so any start of an array will do
+@pytest.mark.parametrize("logN,bits", [(9, 55), (13, 56)])
+def test_transform_between_16_byte_boundaries_stays_in_place(logN, bits):
+    import torch
+    g = context(logN=logN, L=2, bits=bits)
+    pool = Pool()
+    even = torch.stack([torch.arange(g.N, device="cuda") * (i + 7) for i in range(4)])
+    odd = torch.zeros(even.numel() + 1, dtype=torch.int64, device="cuda")[1:].view_as(even)
+    odd.copy_(even)
+    assert odd.data_ptr() % 16 == 8
+    for f in (g.ntt_forward, g.ntt_inverse):
+        f(even, 0, 2)
+        before = pool.get()
+        pool.reset_high()
+        f(odd, 0, 2)
+        assert pool.get(USED_HIGH) <= before
+        assert torch.equal(odd, even)
