@@ -269,8 +269,10 @@ typedef struct ss_batch ss_batch;
 ss_status ss_batch_create(ss_ctx* const* ctxs, int32_t nctx, const ss_batch_item* items, int32_t n, ss_batch** out);
 /* chunk: ciphertexts per pass; nstreams: 1..8 streams, each issuing its own
  * launches, or 0: merged lanes (each chunk a host thread with its own stream;
- * the transforms of all lanes, of rings N >= 8192, run together as one
- * persistent launch per phase over all their tiles); ntt_tile_log: 11 or 12
+ * the transforms of all lanes, of rings N >= 8192 on primes of up to 55 bits,
+ * run together as one persistent launch per phase over all their tiles, and
+ * the inner products of all lanes as one launch; other transforms run on the
+ * lanes' own streams side by side); ntt_tile_log: 11 or 12
  * (words per transform tile, for rings N >= 8192 on primes of more than 55
  * bits; other transforms have one tile size). Kernel timing does not cover
  * merged lanes. */
