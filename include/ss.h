@@ -280,7 +280,8 @@ ss_status ss_batch_config(ss_batch* b, int32_t chunk, int32_t nstreams, int32_t 
 ss_status ss_batch_get_config(const ss_batch* b, int32_t* chunk, int32_t* nstreams, int32_t* ntt_tile_log,
                               int32_t* groups, int32_t* skipped);
 /* Autotuner: times the run for chunk in {8, 32, 64} x streams in {1, 3, 0 (merged lanes)} x tile in
- * {2^11, 2^12} words on this work list and keeps the fastest setting. Synchronous. */
+ * {2^11, 2^12} words on this work list and keeps the fastest setting; the tile stays as configured where no
+ * pair's context has a choice of it (ss_batch_config). Synchronous. */
 ss_status ss_batch_tune(ss_batch* b, ss_stream stream, int32_t* best_chunk, int32_t* best_streams,
                         int32_t* best_tile_log);
 /* Captures the whole run (current setting) as one CUDA graph on `stream` (not the legacy stream). */

@@ -23,6 +23,7 @@
 #include <map>
 #include <mutex>
 #include <thread>
+#include <vector>
 
 #include "ss_internal.h"
 
@@ -426,7 +427,11 @@ ss_status ss_batch_tune(ss_batch* b, ss_stream stream, int32_t* best_chunk, int3
     ss::drop_graph(*b);
     const int chunks[] = {8, 32, 64};
     const int nstr[] = {1, 3, 0};  // 0: merged lanes
-    const int tiles[] = {11, 12};
+    // the tile is a choice only for transforms in the Shoup form
+    const bool wide = std::any_of(b->groups.begin(), b->groups.end(), [&](const ss_batch::Group& g) {
+      return b->ctxs[g.ctx]->N >= 8192 && !b->ctxs[g.ctx]->d_tp;
+    });
+    const std::vector<int> tiles = wide ? std::vector<int>{11, 12} : std::vector<int>{b->tile_log};
     double best = 1e300;
     int bc = b->chunk, bs = b->merged ? 0 : b->nstreams, bt = b->tile_log;
     cudaEvent_t e0, e1;

@@ -68,3 +68,30 @@ def test_lanes_of_both_widths_beside_each_other():
     pairs, refs = products(world, [0, 1, 2, 3, 1], 7)
     _, words = launches_of(world, pairs)
     assert all((w == r).all() for w, r in zip(words, refs))
+
+
+@pytest.mark.parametrize("bits,tiles", [(55, 1), (56, 2)])
+def test_the_tuner_runs_each_different_setting_twice(bits, tiles):
+    """The transform's tile is a choice on primes of more than 55 bits only; elsewhere the tuner leaves it as it was."""
+    import torch
+
+    import paper_2604_19890_gb300 as ssg
+    world = [pair("2N", 13, bits)]
+    pairs, _ = products(world, [0] * 9, bits)
+    g = world[0][0]
+    b = ssg.Batch([g], pairs)
+    st = torch.cuda.Stream()
+    n = 0
+    for chunk in (8, 32, 64):
+        for streams in (1, 3, 0):
+            b.config(chunk, streams)
+            n0 = g.launches()
+            b.run(st)
+            st.synchronize()
+            n += g.launches() - n0
+    b.config(8, 1, 12)
+    n0 = g.launches()
+    best = b.tune(st)
+    assert g.launches() - n0 == 2 * tiles * n
+    assert best[2] == 12 or tiles > 1
+    b.close()
