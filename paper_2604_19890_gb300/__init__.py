@@ -130,7 +130,8 @@ QUERY_STAGES = ["reduction", "comparison", "aggregation", "modulus_raising", "ma
 
 def alu_probe(kind, iters=4096):
     """Integer-pipe ceiling on the current device: kind 0 = 32-bit IMAD/s,
-    kind 1 = 64-bit Shoup forward butterflies/s (registers only)."""
+    kind 1 = forward butterflies/s in the transforms' own form, products by
+    halves (registers only), kind 2 = 32 x 32 -> 64-bit multiply-adds/s."""
     out = C.c_double()
     _chk(lib().ss_alu_probe(int(kind), int(iters), C.byref(out)))
     return out.value

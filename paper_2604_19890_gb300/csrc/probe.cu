@@ -1,8 +1,8 @@
 // Integer-pipe ceilings for the roofline of the ALU-bound kernels: register-only
 // loops that issue the arithmetic of the transforms with no memory traffic.
 //   kind 0: 32-bit multiply-adds (IMAD) per second;
-//   kind 1: forward butterflies per second in Harvey's form: reduce the upper
-//           input below 2q, one 64-bit Shoup product, lazy add and subtract;
+//   kind 1: forward butterflies per second as the transforms on primes up to 55
+//           bits run them: one product by halves (half_mul), one sum, one difference;
 //   kind 2: 32 x 32 -> 64-bit widening multiply-adds (IMAD.WIDE) per second,
 //           the partial products a 64-bit modular product is built from.
 // One full wave of CTAs (as many per SM as fit) runs the loop.
@@ -47,20 +47,19 @@ __global__ void __launch_bounds__(256) k_probe_wide(u64* out, int iters, uint32_
   out[tid] = x;
 }
 
-__global__ void __launch_bounds__(256) k_probe_butterfly(u64* out, int iters, u64 q, u64 w, u64 wp) {
+__global__ void __launch_bounds__(256) k_probe_butterfly(u64* out, int iters, u64 q, u64 w0, u64 w1, uint32_t p0,
+                                                         uint32_t p1) {
   const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
   u64 x[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) x[k] = (tid * 16u + k) % q;
-  const u64 q2 = 2 * q;
-  for (int i = 0; i < iters; ++i) {
+  const u64 nq2 = 0 - 2 * q;
+  for (int i = 0; i < iters; ++i) {  // the words grow without a bound and wrap: only their rate counts
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      u64 U = x[k];
-      if (U >= q2) U -= q2;
-      const u64 V = shoup_lazy(x[k + 8], w, wp, q);
-      x[k] = U + V;
-      x[k + 8] = U - V + q2;
+      const u64 U = x[k], t = half_mul(x[k + 8], w0, w1, p0, p1, nq2);
+      x[k] = U + t;
+      x[k + 8] = U - t;
     }
   }
   u64 s = 0;
@@ -90,14 +89,15 @@ double alu_probe(int kind, int iters) {
   cudaEvent_t e0, e1;
   SS_CUDA(cudaEventCreate(&e0));
   SS_CUDA(cudaEventCreate(&e1));
-  // a 55-bit prime and a twiddle with its Shoup companion, as in the transforms
-  const u64 q = 36028797018652673ULL, w = 12345678901234567ULL % q;
-  const u64 wp = (u64)(((unsigned __int128)w << 64) / q);
+  // a 55-bit modulus and a twiddle with its companions, as in the transforms (half_mul)
+  const u64 q = 36028797018652673ULL, w0 = 12345678901234567ULL % q;
+  const u64 w1 = (u64)(((unsigned __int128)w0 << 32) % q);
+  const uint32_t p0 = (uint32_t)(((unsigned __int128)w0 << 31) / q), p1 = (uint32_t)(((unsigned __int128)w1 << 31) / q);
   float ms = 0;
   for (int rep = 0; rep < 2; ++rep) {  // the first pass warms up
     SS_CUDA(cudaEventRecord(e0, st));
     if (kind == 0) k_probe_imad<<<blocks, threads, 0, st>>>((uint32_t*)buf, iters, 0x9E3779B9u);
-    else if (kind == 1) k_probe_butterfly<<<blocks, threads, 0, st>>>((u64*)buf, iters, q, w, wp);
+    else if (kind == 1) k_probe_butterfly<<<blocks, threads, 0, st>>>((u64*)buf, iters, q, w0, w1, p0, p1);
     else k_probe_wide<<<blocks, threads, 0, st>>>((u64*)buf, iters, 0x9E3779B9u);
     SS_CUDA(cudaEventRecord(e1, st));
     SS_CUDA(cudaEventSynchronize(e1));
