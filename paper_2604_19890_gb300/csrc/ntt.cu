@@ -1374,7 +1374,7 @@ NttArgs make_args(Context& C, const PolySet& s) {
   A.mods = reinterpret_cast<const Modulus*>(C.d_mod);
   A.tw = C.d_tw;
   A.tp = C.d_tp;
-  A.tws = C.N + (C.N >> chunk_log(C));
+  A.tws = C.d_tp ? ntt_tw_slots(C) : 0;
   A.ninv = C.d_ninv;
   A.split = C.d_split;
   A.src = nullptr;
