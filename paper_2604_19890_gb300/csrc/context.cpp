@@ -642,6 +642,9 @@ void build_context(Context& C, const ss_params& prm) {
     for (int it = 0; it < 5; ++it) x *= 2 - q * x;
     md[i].qinv = 0 - x;
   }
+  int dev = 0;
+  SS_CUDA(cudaGetDevice(&dev));
+  SS_CUDA(cudaDeviceGetAttribute(&C.sms, cudaDevAttrMultiProcessorCount, dev));
   upload((void**)&C.d_mod, md.data(), sizeof(ModDesc) * T);
 
   std::vector<u64> r64(kR64 * T, 0), fold_w1(T, 1);  // fold_w1: the forward node-1 twiddle of X^N + 1

@@ -1453,7 +1453,7 @@ void k_modup(Context& C, const u64* src, u64* dst, int level, int B, cudaStream_
   const int bx = (C.N + 2 * TPB - 1) / (2 * TPB);
   // four blocks of 256 threads per SM, a part of four targets at least
   const long blocks = (long)bx * dn * B;
-  A.parts = (int)std::max(1L, std::min((4L * 152 + blocks - 1) / blocks, (long)nx / 4));
+  A.parts = (int)std::max(1L, std::min((4L * C.sms + blocks - 1) / blocks, (long)nx / 4));
   const dim3 g(bx, dn * A.parts, B);
   const size_t smem = (size_t)((nx + A.parts - 1) / A.parts + 1) * (2 * a + 2) * 8;
   if (B > 65535 || dn * A.parts > 65535) throw Error(SS_ERR_SHAPE, "too many digits or ciphertexts in one conversion");
@@ -1659,7 +1659,8 @@ void k_lift_small(Context& C, const i64* e, const u64* m, u64 tmul, u64* out, lo
                   int q0, int nq, cudaStream_t st) {
   // all limbs in one thread, or fewer where that leaves SMs without blocks
   const dim3 b = grid_for(C.N / 2, n_outer);
-  const int parts = (int)std::min((long)nl, std::max(1L, (8L * 152 + b.x * (long)b.y - 1) / (b.x * (long)b.y)));
+  const long blocks = (long)b.x * b.y;
+  const int parts = (int)std::min((long)nl, std::max(1L, (8L * C.sms + blocks - 1) / blocks));
   const int per = (nl + parts - 1) / parts;
   launch_early(k_lift_small_impl, dim3(b.x, b.y, (nl + per - 1) / per), TPB, 0, st, e, m, tmul, out, out_os, nl, per, q0,
                nq, C.L, C.N, C.d_mod);

@@ -1281,9 +1281,9 @@ __global__ void __launch_bounds__(128, 6) k_ntt16_multi(const __grid_constant__ 
 
 // column phase of one transform by halves
 template <bool FWD, int LOGS, int LOG2N, int RING>
-void launch_cols_as(int npoly, cudaStream_t st, const NttArgs& A) {
+void launch_cols_as(int sms, int npoly, cudaStream_t st, const NttArgs& A) {
   constexpr int CL = kColTile - LOGS, CLB = kColTileBig - LOGS;
-  if (((long)npoly << (LOGS + LOG2N - kColTileBig)) >= 2L * SS_COLS_BIG * 152)
+  if (((long)npoly << (LOGS + LOG2N - kColTileBig)) >= 2L * SS_COLS_BIG * sms)
     launch_early(k_ntt16_cols<FWD, LOGS, LOG2N, CLB, RING>, dim3(1 << (LOG2N - CLB), npoly), 256,
                  col_smem<LOGS, CLB>(), st, A);
   else
@@ -1291,22 +1291,22 @@ void launch_cols_as(int npoly, cudaStream_t st, const NttArgs& A) {
                  A);
 }
 template <bool FWD>
-void launch_cols(int ring, int logS, int log2n, int npoly, cudaStream_t st, const NttArgs& A) {
-  switch (ring * 16 + logS) {
-    case 16 + 5: launch_cols_as<FWD, 5, 8, 1>(npoly, st, A); break;
-    case 16 + 6: launch_cols_as<FWD, 6, 8, 1>(npoly, st, A); break;
-    case 16 + 7: launch_cols_as<FWD, 7, 8, 1>(npoly, st, A); break;
-    case 16 + 8: launch_cols_as<FWD, 8, 8, 1>(npoly, st, A); break;
-    case 48 + 5: launch_cols_as<FWD, 5, 8, 3>(npoly, st, A); break;
-    case 48 + 6: launch_cols_as<FWD, 6, 8, 3>(npoly, st, A); break;
-    case 48 + 7: launch_cols_as<FWD, 7, 8, 3>(npoly, st, A); break;
-    case 48 + 8: launch_cols_as<FWD, 8, 8, 3>(npoly, st, A); break;
+void launch_cols(const Context& C, int logS, int log2n, int npoly, cudaStream_t st, const NttArgs& A) {
+  switch (C.m_odd * 16 + logS) {
+    case 16 + 5: launch_cols_as<FWD, 5, 8, 1>(C.sms, npoly, st, A); break;
+    case 16 + 6: launch_cols_as<FWD, 6, 8, 1>(C.sms, npoly, st, A); break;
+    case 16 + 7: launch_cols_as<FWD, 7, 8, 1>(C.sms, npoly, st, A); break;
+    case 16 + 8: launch_cols_as<FWD, 8, 8, 1>(C.sms, npoly, st, A); break;
+    case 48 + 5: launch_cols_as<FWD, 5, 8, 3>(C.sms, npoly, st, A); break;
+    case 48 + 6: launch_cols_as<FWD, 6, 8, 3>(C.sms, npoly, st, A); break;
+    case 48 + 7: launch_cols_as<FWD, 7, 8, 3>(C.sms, npoly, st, A); break;
+    case 48 + 8: launch_cols_as<FWD, 8, 8, 3>(C.sms, npoly, st, A); break;
     case 80 + 6:
-      if (log2n == 7) launch_cols_as<FWD, 6, 7, 5>(npoly, st, A);
-      else launch_cols_as<FWD, 6, 8, 5>(npoly, st, A);
+      if (log2n == 7) launch_cols_as<FWD, 6, 7, 5>(C.sms, npoly, st, A);
+      else launch_cols_as<FWD, 6, 8, 5>(C.sms, npoly, st, A);
       break;
-    case 80 + 7: launch_cols_as<FWD, 7, 8, 5>(npoly, st, A); break;
-    default: launch_cols_as<FWD, 8, 8, 5>(npoly, st, A); break;
+    case 80 + 7: launch_cols_as<FWD, 7, 8, 5>(C.sms, npoly, st, A); break;
+    default: launch_cols_as<FWD, 8, 8, 5>(C.sms, npoly, st, A); break;
   }
 }
 
@@ -1476,12 +1476,12 @@ static void launch(Context& C, const PolySet& s, bool fwd, cudaStream_t st, cons
         A1.src_os = src_os;
       }
       if (fwd) {
-        launch_cols<true>(C.m_odd, log1, log2n, npoly, st, A);
+        launch_cols<true>(C, log1, log2n, npoly, st, A);
         launch_rows<true, false>(log2n, s, st, A);
       } else {
         if (src) launch_rows<false, true>(log2n, s, st, A1);
         else launch_rows<false, false>(log2n, s, st, A);
-        launch_cols<false>(C.m_odd, log1, log2n, npoly, st, A);
+        launch_cols<false>(C, log1, log2n, npoly, st, A);
       }
     } else if (fwd) {
       if (C.m_odd == 3) launch16<true, true, false, false, 3>(log1, g1, thr, smem(tile), st, A, logc1, 1);
@@ -1606,7 +1606,7 @@ void ntt_forward_cols(Context& C, const PolySet& s, cudaStream_t st) {
   if (npoly == 0) return;
   if (npoly > 65535) throw Error(SS_ERR_SHAPE, "too many polynomials in one transform");
   int kr = kt_begin(C, st);
-  launch_cols<true>(C.m_odd, C.logN - l2, l2, npoly, st, make_args(C, s));
+  launch_cols<true>(C, C.logN - l2, l2, npoly, st, make_args(C, s));
   ++C.launches;
   if (kr >= 0) C.kt.ntt_products += ntt_products(C, s, true);
   kt_end(C, kr, KC_NTT, 16.0 * C.N * active_polys(s), st);
@@ -1656,7 +1656,7 @@ void rows_ip(Context& C, const RowsIpReq& R, cudaStream_t st) {
   // the rows' threads; a grid that leaves room gets 256 a CTA for the sums, whose
   // loads are then one round deep (rotations near the chain's end: 815 -> 610 us)
   int thr = (A.nb * rpc * tpr + 31) / 32 * 32;
-  if ((long)g.x * g.y <= SS_ROWS_IP * 152L) thr = 256;
+  if ((long)g.x * g.y <= (long)SS_ROWS_IP * C.sms) thr = 256;
   const size_t smem = ((size_t)24 << l2) + (size_t)(thr / tpr) * 8 * (1 << l2);
   const double words = (double)A.dn * R.nlimbs * (R.B + 2.0) +
                        (R.type == 0 ? 2.0 : 4.0 + (R.x ? 2.0 : 0.0)) * R.nlimbs * R.B;

@@ -135,6 +135,7 @@ struct Context {
   u64 gr_w[2] = {0, 0}, theta4[4] = {0, 0, 0, 0};
   std::vector<std::pair<int, int>> gens;  // slot-group generators mod M' with their orders
 
+  int sms = 0;  // SMs of the device the context was made on: grids are dealt by it
   // device tables
   ModDesc* d_mod = nullptr;           // [ntot]
   u64* d_tw = nullptr;                // per prime 4N words: forward (w, shoup) pairs, then inverse ones; products by
