@@ -347,8 +347,7 @@ ss_status ss_set_batch(ss_ctx* ctx, int32_t batch);
 /* ---- raw transform (for kernel-level measurement) ---- */
 /* In-place NTT over the context's ring of `npoly` consecutive limbs of N words; limb k uses
  * data prime (first_prime + k % nprimes). Input words must be residues below
- * their prime (the forward transform keeps lazy sums below 40q, which needs
- * inputs below 4q); outputs are residues below the prime, forward in the
+ * their prime (the forward transform's lazy sums need inputs below 4q); outputs are residues below the prime, forward in the
  * evaluation order given above. */
 ss_status ss_ntt_forward(ss_ctx* ctx, uint64_t* data, int32_t npoly, int32_t first_prime, int32_t nprimes,
                          ss_stream stream);
@@ -377,9 +376,9 @@ ss_status ss_kernel_stats(ss_ctx* ctx, int32_t cls, uint64_t* launches, double* 
 
 /* Products (one 64-bit modular product by a precomputed constant each) that the
  * timed transforms performed, those finished inside the fused inner product
- * included, since kernel timing was switched on: per polynomial N/2 log2 N forward, less N/2 when the base conversion
- * that wrote the input already applied the first stage's twiddle (ring
- * X^N + 1), and N/2 (log2 N + 1) inverse for N > 4096 (the last stage also
+ * included, since kernel timing was switched on: per polynomial N/2 log2 N
+ * forward, less N/2 when the base conversion that wrote the input already
+ * applied the first stage's twiddle (ring X^N + 1), and N/2 (log2 N + 1) inverse for N > 4096 (the last stage also
  * scales the sums by N^-1), N/2 (log2 N + 2) for N <= 4096 (N^-1 on every
  * word), N/2 (log2 N - 1) when the last stage's factors are left to the base
  * conversion that reads the output (ring X^N + 1, N > 4096). The

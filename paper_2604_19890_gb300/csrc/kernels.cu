@@ -237,11 +237,12 @@ __device__ __forceinline__ void sum_halves(const u32 (&yl)[NS][V], const u32 (&y
 // dst limb m (global prime g(m) = m < nq ? m : L + m - nq), m outside
 // [skip_lo, skip_hi):  sum_s [src_s * c1_s]_{q_s} * c2[s][g(m)]  (mod q_g), then
 // times post[g] when post != null. Source s lives on prime sp0 + s (s < nsq)
-// or L + s - nsq. Words come out below 2q (the single-phase transform's folded first
-// stage subtracts them from 2q): sum_s of the halves' products is below NS (2^SPLIT +
-// 2^(bits-SPLIT)) q <= 2^32 q, a Montgomery step by 2^32 leaves below that plus q. NS <= 4
-// sources, halves of y_s and one Montgomery step by 2^32 as in k_modup; SPLIT low bits keep the low products' sum below 2^64 also for
-// 58-bit primes (8 (2^29 - 1)(2^32 - 1) for NS = 4). Per block, each target's
+// or L + s - nsq. NS <= 4 sources, halves of y_s and one Montgomery step by 2^32 as
+// in k_modup. Words come out below 2q (the single-phase transform's folded first
+// stage subtracts them from 2q): the halves' products sum to less than NS (2^SPLIT +
+// 2^(bits-SPLIT)) q <= 2^32 q, of which the Montgomery step leaves less than q, plus q
+// at most. SPLIT low bits keep the low products' sum below 2^64 also for 58-bit
+// primes (8 (2^29 - 1)(2^32 - 1) for NS = 4). Per block, each target's
 // modulus, -q^-1 mod 2^64 and the pairs (c2 post 2^32, c2 post 2^(32+SPLIT)) mod
 // q_g are staged once in shared memory (row m: q, -q^-1, the pairs), one thread a
 // pair. (128-bit sums and a Montgomery step by 2^64 kept the multiply pipe 81 %
@@ -416,13 +417,13 @@ __global__ void __launch_bounds__(256) k_bconv_many_impl(const u64* src, long sr
 // l)) converted to the other data primes and the special primes, for every digit
 // in one launch. Output word: sum_s y_s c_s mod q_g, y_s = [x_s c1_s]_{q_s} exact.
 // By halves of y_s (SPLIT low bits l_s, the rest h_s): sum_s l_s c_s0 + h_s c_s1 with
-// c_s0 = c_s 2^32, c_s1 = c_s 2^(32+SPLIT) mod q_g, below (NS / 4 + ..) 2^32 q_g < 2^32 q_g, and one
-// Montgomery step by 2^32; the result is below 2 q_g, as the forward transform that
-// reads it takes. SPLIT leaves the low products' sum below 2^64, so a target costs
+// c_s0 = c_s 2^32, c_s1 = c_s 2^(32+SPLIT) mod q_g, below NS (2^SPLIT + 2^(bits-SPLIT)) q_g
+// < 2^32 q_g, and one Montgomery step by 2^32; the result is below 2 q_g, as the forward
+// transform that reads it takes. SPLIT leaves the low products' sum below 2^64, so a target costs
 // 4 NS + 2 accumulating 64-bit products and one 32-bit one (58 cycles of the multiply
 // pipe a warp for NS = 3) where 128-bit sums and a Montgomery step by 2^64 took 72 and
 // 128-bit carries. The constants come from a table made with the context
-// (ModupTab), the upper half's already times the transform's node-1 twiddle.
+// (Context::d_modup), the upper half's already times the transform's node-1 twiddle.
 // One launch per digit left most SMs idle for few ciphertexts or small rings (two
 // ciphertexts at N = 2^16: 256 blocks of the 1216 that fit); when even all digits
 // do not fill the GPU, the targets of a digit are dealt to `parts` blocks.
@@ -858,8 +859,9 @@ __global__ void k_uniform_impl(u64* out, long out_os, int nl, int q0, int nq, in
 
 // Encryption's last step, limb i of ciphertext o: c1 = uniform (the words of
 // k_uniform_impl), c0 = c0 - c1 s. One pass instead of writing c1 and reading it back.
-__global__ void __launch_bounds__(256) k_enc_tail_impl(u64* c0, u64* c1, long os, int L, u32 id0, u32 tag, u32 k0, u32 k1,
-                                                       const u64* s, int N, const ModDesc* mods, const u64* r64) {
+__global__ void __launch_bounds__(256) k_enc_tail_impl(u64* c0, u64* c1, long os, int L, u32 id0, u32 tag, u32 k0,
+                                                       u32 k1, const u64* s, int N, const ModDesc* mods,
+                                                       const u64* r64) {
   enter_grid();
   const int i = blockIdx.y % L, o = blockIdx.y / L;
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1312,9 +1314,8 @@ void k_lincomb(Context& C, const std::vector<const Buf*>& ys, const std::vector<
   int polys = out.count * out.ncomp * out.level;
   TIMED(KC_ELEM, (nt + 1.0) * polys * C.N * 8.0,
         launch_early(k_lincomb_impl, grid_for(C.N / 2, polys), TPB, 0, st,
-                     A, nt, cst, small ? npos + 1 : 0, tiny ? 1 : 0, out.data,
-                                                                  out.cap, C.N,
-                                                              out.ncomp, out.level, C.d_mod));
+                     A, nt, cst, small ? npos + 1 : 0, tiny ? 1 : 0, out.data, out.cap, C.N, out.ncomp, out.level,
+                     C.d_mod));
   LAUNCHED();
 }
 
@@ -1375,8 +1376,8 @@ void k_lincomb_multi(Context& C, const std::vector<const Buf*>& ys, const std::v
 }
 
 void k_batch_sum(Context& C, const Buf& a, Buf& out, cudaStream_t st) {
-  launch_early(k_batch_sum_impl, grid_for(C.N, a.ncomp * a.level), TPB, 0, st, a.data, out.data, a.count, a.ncomp, a.level,
-                                                                      a.cap, out.cap, C.N, C.d_mod);
+  launch_early(k_batch_sum_impl, grid_for(C.N, a.ncomp * a.level), TPB, 0, st, a.data, out.data, a.count, a.ncomp,
+               a.level, a.cap, out.cap, C.N, C.d_mod);
   ++C.launches;
   SS_CUDA(cudaGetLastError());
 }
@@ -1395,8 +1396,8 @@ void k_binary(Context& C, int op, const Buf& a, const Buf& b, Buf& out, cudaStre
 void k_scalar(Context& C, int op, const Buf& a, i64 c, Buf& out, cudaStream_t st) {
   int polys = a.count * a.ncomp * a.level;
   TIMED(KC_ELEM, 2.0 * polys * (double)C.N * 8.0,
-  launch_early(k_scalar_impl, grid_for(C.N / 2, polys), TPB, 0, st, op, a.data, c, out.data, C.N, a.ncomp, a.level, a.cap,
-                                                       out.cap, C.d_mod, C.d_pinv));
+  launch_early(k_scalar_impl, grid_for(C.N / 2, polys), TPB, 0, st, op, a.data, c, out.data, C.N, a.ncomp, a.level,
+               a.cap, out.cap, C.d_mod, C.d_pinv));
   LAUNCHED();
 }
 
@@ -1662,8 +1663,8 @@ void k_lift_small(Context& C, const i64* e, const u64* m, u64 tmul, u64* out, lo
   const long blocks = (long)b.x * b.y;
   const int parts = (int)std::min((long)nl, std::max(1L, (8L * C.sms + blocks - 1) / blocks));
   const int per = (nl + parts - 1) / parts;
-  launch_early(k_lift_small_impl, dim3(b.x, b.y, (nl + per - 1) / per), TPB, 0, st, e, m, tmul, out, out_os, nl, per, q0,
-               nq, C.L, C.N, C.d_mod);
+  launch_early(k_lift_small_impl, dim3(b.x, b.y, (nl + per - 1) / per), TPB, 0, st, e, m, tmul, out, out_os, nl, per,
+               q0, nq, C.L, C.N, C.d_mod);
   LAUNCHED();
 }
 
@@ -1677,8 +1678,8 @@ void k_mul_sub(Context& C, const u64* x, long x_os, const u64* a, long a_os, con
 void k_enc_tail(Context& C, u64* c0, u64* c1, long os, int n_outer, u32 id0, u32 tag, cudaStream_t st) {
   u32 k0, k1;
   seed_words(C, k0, k1);
-  launch_early(k_enc_tail_impl, grid_for(C.N, n_outer * C.L), TPB, 0, st, c0, c1, os, C.L, id0, tag, k0, k1, C.d_sk, C.N,
-               C.d_mod, C.d_r64);
+  launch_early(k_enc_tail_impl, grid_for(C.N, n_outer * C.L), TPB, 0, st, c0, c1, os, C.L, id0, tag, k0, k1, C.d_sk,
+               C.N, C.d_mod, C.d_r64);
   LAUNCHED();
 }
 

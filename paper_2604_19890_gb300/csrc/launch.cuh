@@ -8,9 +8,9 @@
 // predecessor, so the order is the stream's order throughout). Kernels without
 // enter_grid are launched the plain way and wait for complete predecessors.
 // The key switch of a small ring is a chain of a dozen kernels of a few
-// microseconds each, whose launch gaps this hides: with one scratch block per key
-// switch and no copy of the product, one multiplication at N = 2^13 took 76 us
-// instead of 90, a query there 4.47 ms instead of 5.03. Blocks that wait early hold
+// microseconds each, whose launch gaps this hides: by itself it takes a query at
+// N = 2^13 from 4.50 ms to 4.19, a rotate-sum at N = 2^15 from 652 us to 611 and one
+// multiplication at N = 2^13 from 69.6 us to 68.6. Blocks that wait early hold
 // room that kernels of other streams could use, so a thread that feeds one of
 // several streams side by side launches the plain way (PlainLaunches): the mixed
 // batch on three streams took 11.1 ms with early launches and 10.8 without.

@@ -11,7 +11,8 @@
 // A length-N transform is split N = N1 * N2. Its first log2(N1) stages act on
 // the N2 columns (stride N2) independently, the remaining log2(N2) stages on
 // the N1 contiguous chunks of N2 words. Each phase is one kernel whose CTAs hold
-// 2048-word tiles in registers and shared memory. N <= 4096 runs in one phase.
+// tiles of 2048 or 4096 words in registers and shared memory. N <= 4096 runs in
+// one phase.
 // Three forms, by size and prime width:
 //  * N >= 8192, primes below 2^55: k_ntt16_cols / k_ntt16_rows (products by
 //    halves, below). One GB300, 328 limbs of 2^16 words: 0.565 us a limb forward
@@ -43,7 +44,9 @@ constexpr int TILE = 4096;  // words per CTA tile (32 KiB of shared memory)
 #ifndef SS_NTT_MINB_I
 #define SS_NTT_MINB_I 3
 #endif
-// resident CTAs of 128 threads per SM that the phases of products by halves are compiled for
+// resident CTAs of 128 threads per SM that the phases of products by halves are compiled for (72 registers, 64 in
+// the large column tiles and the fused inner product; they spill 4 to 60 bytes a thread for it. 328 limbs of 2^16
+// words, us a limb forward / inverse at 5, 6, 7, 8 CTAs: 0.579/0.607, 0.569/0.593, 0.565/0.573, 0.576/0.587)
 #ifndef SS_COLS_F
 #define SS_COLS_F 7
 #endif
@@ -190,7 +193,9 @@ __device__ __forceinline__ u64 reduce_half(u64 v, const HalfMod& m) {
 // quadratics share the products c_1 a3 and c_1 (a2 + a3); each remainder is
 // then evaluated at its two roots. Forward: 6 Shoup products per 4 words,
 // inputs below 4q give outputs below 16q, in the order xi^1, xi^3, xi^7, xi^9.
-// Inverse (inputs below off, a multiple of q with 2 off + q < 2^64): the remainders from the root values, then
+// Inverse (inputs below B; off a multiple of q, B <= off and B + off + 2q < 2^64:
+// every difference lifted by off or off + q stays in one positive word): the
+// remainders from the root values, then
 // a3 = (r0 - s0) / (1 - 2 c_1), a2 + a3 = (s1 - r1) / (1 - 2 c_1),
 // a1 = r1 - c_1 (a2 + a3), a0 = r0 + a2 + c_1 a3, scaled by 4/N: 10 products,
 // canonical. Constants per prime (value, Shoup pairs): forward c_1, xi, xi^3,
@@ -332,7 +337,8 @@ __global__ void __launch_bounds__(512) k_ntt(NttArgs A, int logS, int logCPB, in
   __syncthreads();
   // m = 5N/2 (one phase over CPB = 4 chunks, the four factors): the split
   // first, residues brought below 2q for the rounds
-  const ulonglong2* spl = RING == 5 ? reinterpret_cast<const ulonglong2*>(A.split + (size_t)pidx * kSplitWords) : nullptr;
+  const ulonglong2* spl =
+      RING == 5 ? reinterpret_cast<const ulonglong2*>(A.split + (size_t)pidx * kSplitWords) : nullptr;
   if (RING == 5 && FWD) {
     const int n4 = W >> 2;
     for (int i = tid; i < n4; i += T) {
@@ -598,7 +604,7 @@ __device__ __forceinline__ void ntt16_tile(const NttArgs& A, int logCPB, int m0,
                   const u64 t = shoup_lazy(V, w, wp, q);
                   x[k] = U + t;
                   x[k + d] = U + V + q2 - t;
-                } else if (pre1) {  // U, V < q
+                } else if (pre1) {  // U, V < 2q, as a base conversion leaves them
                   x[k] = U + V;
                   x[k + d] = U - V + q2;
                 } else if (FWD) {
@@ -811,8 +817,8 @@ __device__ __forceinline__ void ntt16_cols(const NttArgs& A, int tile, int poly)
       for (int j = 4 - NS; j < JE; ++j) half_stage<false>(x, j, j - (4 - NS), twS, tpS, hm, false, wide_slot);
     }
     const u64* nv = A.ninv + 6 * pidx;
-    const u64 off = q << (5 + NS - 1);  // above every input of the last stage
-    if (RING == 5) {
+    const u64 off = q << (5 + NS - 1);  // no input of the last stage is above it
+    if (RING == 5) {  // the split takes two stages: its inputs are below off / 2 <= 128q
 #pragma unroll
       for (int k = 0; k < 4; ++k) split4_inv(x[k], x[k + 4], x[k + 8], x[k + 12], spl, q, off);
     } else if (RING == 3) {
@@ -858,7 +864,8 @@ constexpr size_t col_smem() {
 }
 
 template <bool FWD, int LOGS, int LOG2N, int CL, int RING>
-__global__ void __launch_bounds__(1 << (LOGS + CL - 4), LOGS + CL == kColTile ? (FWD ? SS_COLS_F : SS_COLS_I) : SS_COLS_BIG)
+__global__ void __launch_bounds__(1 << (LOGS + CL - 4),
+                                  LOGS + CL == kColTile ? (FWD ? SS_COLS_F : SS_COLS_I) : SS_COLS_BIG)
     k_ntt16_cols(NttArgs A) {
   enter_grid();
   ntt16_cols<FWD, LOGS, LOG2N, CL, RING>(A, blockIdx.x, blockIdx.y);
@@ -1006,7 +1013,8 @@ __device__ __forceinline__ void ntt16_rows(const NttArgs& A, const RowPlan& R, i
 #pragma unroll
       for (int i = 0; i < S / 64; ++i) {
         const int r = 2 * (lane + 32 * i);
-        if (ok) *reinterpret_cast<ulonglong2*>(rp + r) = *reinterpret_cast<const ulonglong2*>(data + rw * S + row_swz(r));
+        if (ok)
+          *reinterpret_cast<ulonglong2*>(rp + r) = *reinterpret_cast<const ulonglong2*>(data + rw * S + row_swz(r));
       }
     }
   } else {
@@ -1129,7 +1137,8 @@ __global__ void __launch_bounds__(256, SS_ROWS_IP) k_rows_ip(const __grid_consta
   u64 x[16];
   if (valid) {
     const int b = row / rpc, r = row - b * rpc;
-    const u64* src = r < nd ? A.ext + (long)(b0 + b) * A.ext_os + (long)(r + (r >= own ? 1 : 0)) * (A.level + A.alpha) * A.N
+    const long digit = r + (r >= own ? 1 : 0);
+    const u64* src = r < nd ? A.ext + (long)(b0 + b) * A.ext_os + digit * (A.level + A.alpha) * A.N
                             : A.delta + ((long)(b0 + b) * 2 + (r - nd)) * A.nl * A.N;
     src += limb + lr;
 #pragma unroll
@@ -1287,8 +1296,8 @@ void launch_cols_as(int sms, int npoly, cudaStream_t st, const NttArgs& A) {
     launch_early(k_ntt16_cols<FWD, LOGS, LOG2N, CLB, RING>, dim3(1 << (LOG2N - CLB), npoly), 256,
                  col_smem<LOGS, CLB>(), st, A);
   else
-    launch_early(k_ntt16_cols<FWD, LOGS, LOG2N, CL, RING>, dim3(1 << (LOG2N - CL), npoly), 128, col_smem<LOGS, CL>(), st,
-                 A);
+    launch_early(k_ntt16_cols<FWD, LOGS, LOG2N, CL, RING>, dim3(1 << (LOG2N - CL), npoly), 128,
+                 col_smem<LOGS, CL>(), st, A);
 }
 template <bool FWD>
 void launch_cols(const Context& C, int logS, int log2n, int npoly, cudaStream_t st, const NttArgs& A) {

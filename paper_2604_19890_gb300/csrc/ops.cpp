@@ -114,8 +114,8 @@ static void modup(Context& C, const u64* dc, u64* ext, int l, int B, bool pre, b
     const int lo = j * a, hi = std::min(lo + a, l);
     const u64* c1 = C.d_tables + C.off_modup.at({j, hi});
     const u64* c2 = c1 + 2 * (hi - lo);
-    k_bconv(C, dc + (size_t)lo * N, (long)l * N, hi - lo, lo, c1, c2, ext + (size_t)j * nx * N, (long)dn * nx * N, nx, l,
-            lo, hi, nullptr, B, st, -1, pre, post);
+    k_bconv(C, dc + (size_t)lo * N, (long)l * N, hi - lo, lo, c1, c2, ext + (size_t)j * nx * N, (long)dn * nx * N, nx,
+            l, lo, hi, nullptr, B, st, -1, pre, post);
   }
 }
 
@@ -147,7 +147,8 @@ static void keyswitch_impl(Context& C, const Buf& in, int comp, const KeyDev& K,
   const bool fused = rows_ip_fits(C, l);
   if (fused) {
     ntt_forward_cols(C, ps, st);
-    rows_ip(C, RowsIpReq{0, ext, d, in_os, &K, l, B, l, a, acc, nullptr, false, nullptr, nullptr, nullptr, nullptr}, st);
+    rows_ip(C, RowsIpReq{0, ext, d, in_os, &K, l, B, l, a, acc, nullptr, false, nullptr, nullptr, nullptr, nullptr},
+            st);
   } else {
     ntt_forward(C, ps, st);
     k_ks_ip(C, d, in_os, ext, ext_os, K, l, acc, sp_os, B, st, l, a);
@@ -222,7 +223,8 @@ void op_relin_drop(Context& C, const Buf& in, Buf& out, cudaStream_t st) {
   //    with P d added on q_{l-1}
   const u64* pmod = C.d_tables + C.off_pmod;
   if (fused)
-    rows_ip(C, RowsIpReq{0, ext, d, in_os, &C.rlk, l, B, l - 1, ns, acc, &in, true, nullptr, pmod, nullptr, nullptr}, st);
+    rows_ip(C, RowsIpReq{0, ext, d, in_os, &C.rlk, l, B, l - 1, ns, acc, &in, true, nullptr, pmod, nullptr, nullptr},
+            st);
   else
     k_ks_ip(C, d, in_os, ext, ext_os, C.rlk, l, acc, sp_os, B, st, l - 1, ns, &in, pmod);
   // 4. ModDown by q_{l-1} P: delta = t conv([t^-1 (P d + acc)]_D) on the first l-1 primes

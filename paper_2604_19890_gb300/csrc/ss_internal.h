@@ -142,9 +142,9 @@ struct Context {
                                       //   halves: per prime and direction ntt_tw_slots pairs (w, 2^32 w mod q)
   u32* d_tp = nullptr;                // products by halves (N >= 8192, primes below 2^55): for each pair of d_tw the
                                       //   two half-quotients floor(w 2^31 / q); else null
-  u64* d_r64 = nullptr;               // [ntot][kR64] mod q: 2^64, 2^64 w; 2^64 N^-1, 2^64 N^-1 psi^(-N/2) (the inverse's
-                                      //   last stage); 2^32, 2^32 w; 2^62, 2^62 w; 2^61, 2^61 w, with w the forward
-                                      //   node-1 twiddle psi^(N/2) (entries with w, N^-1: X^N + 1 only)
+  u64* d_r64 = nullptr;               // [ntot][kR64] mod q: 2^64, 2^64 w; 2^64 N^-1, 2^64 N^-1 psi^(-N/2) (the
+                                      //   inverse's last stage); 2^32, 2^32 w; 2^62, 2^62 w; 2^61, 2^61 w, with w the
+                                      //   forward node-1 twiddle psi^(N/2) (entries with w, N^-1: X^N + 1 only)
   u64* d_ninv = nullptr;              // [ntot][6] N^{-1}, shoup, N^{-1} psi^{-N/2} (m = 3N: 2 c), shoup, (m = 3N: c =
                                       //   (2 rho - 1)^{-1} N^{-1}), shoup
   u64* d_split = nullptr;             // m = 5N/2: [ntot][12][2] four-way split constants (forward 5, inverse 7)
@@ -186,7 +186,7 @@ struct Context {
   // evaluator
   int batch = 8;
   bool reduced_g = false;  // evaluate G_{p,e} with the lattice-reduced coefficients
-  int ntt_tile_log = SS_NTT_TILE_LOG;  // words per CTA tile of the two-phase transform: 2^11 or 2^12
+  int ntt_tile_log = SS_NTT_TILE_LOG;  // words per CTA tile of the Shoup form's phases: 2^11 or 2^12
   bool trace_on = false;
   std::vector<std::string> trace;
   std::atomic<unsigned long long> launches{0};  // shared by server worker threads
@@ -228,11 +228,13 @@ struct PlainLaunches {
 // (o % skip_mod) * skip_w .. are skipped when skip_w > 0 (ModUp outputs).
 // pre_w1 (forward, ring X^N + 1): the upper half of every polynomial already
 // carries the node-1 twiddle psi^(N/2) (the base conversion that wrote it
-// applied it), so the first stage adds and subtracts without its product.
+// applied it, words below 2q), so the first stage adds and subtracts without
+// its product.
 // post_scale (inverse, ring X^N + 1, N > 4096): the last stage adds and
 // subtracts without its products and leaves N^-1 (lower half) and
 // N^-1 psi^(-N/2) (upper half) to the consumer, a base conversion that folds
-// them into its per-source constants; the words are then unreduced (< 4q).
+// them into its per-source constants; the words are then unreduced: below 4q in the
+// Shoup form, below 512q by halves, so the consumer must take any 64-bit word.
 struct PolySet {
   u64* base;
   long outer_stride;
